@@ -334,7 +334,7 @@ const char* pic_last_error(const pic_handle* h);
  * application, a plugin inside another framework's memory pool), where a
  * cudaMalloc could fail, block or synchronise the device at the wrong time.
  * The caller passes inputs and outputs; the scratch (a (cell, chunk)
- * histogram) is a fixed 4 MiB device array inside this library that every
+ * histogram and its tile sums) is a fixed 4 MiB device array (and 1 KiB) inside this library that every
  * GPU loading the library holds until the process exits.
  *
  * z..id: n input particles (device); z_out..id_out: n outputs (device), not

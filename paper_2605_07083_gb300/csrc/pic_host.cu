@@ -26,9 +26,12 @@ __global__ void k_profile(DevState st);
 __global__ void k_phi(DevState st);
 __global__ void k_fill_ids(uint32_t* id, long long n, uint32_t first);
 __global__ void k_count_outside(const float* z, long long n, float Lf, int* bad);
-void sort_launch(const DevState& st, int max_chunks, int max_nz, cudaStream_t s);
-size_t sort_hist_ints(const int32_t* seg_cap, const int* seg_nz, int n_seg, int64_t* hoff);
-int sort_max_chunks(const int32_t* seg_cap, int n_seg);
+void sort_launch(const DevState& st, const SortGrid& r, int max_nz, cudaStream_t s);
+int sort_slots(int sms, int n_seg, int max_nz);
+size_t sort_hist_ints(const int32_t* seg_cap, const int* seg_nz, int n_seg, int slots,
+                      int64_t* hoff);
+size_t sort_tiles(size_t hist_ints);
+SortGrid sort_grid(const int32_t* seg_cap, const int* seg_nz, int n_seg, int slots);
 cudaError_t sort_prepare(int smem_bytes);
 }  // namespace pic
 
@@ -84,7 +87,7 @@ struct pic_handle {
   int bw_len = 0;
   int mcc_blocks = 0;
   bool sort_ready = false;
-  int sort_chunks = 1;
+  SortGrid sort_grid{1, 1, 1};
   int prof_gx = 1;              // k_profile blocks per segment
   size_t prof_smem = 0;
   char last_error[256] = {0};
@@ -423,9 +426,10 @@ int sort_alloc(pic_handle* h) {
   std::vector<int> nz(h->n_seg);
   std::vector<int64_t> hoff(h->n_seg);
   for (int g = 0; g < h->n_seg; ++g) nz[g] = h->cfg[g / 3].n_cells;
-  const size_t hist = sort_hist_ints(h->seg_cap.data(), nz.data(), h->n_seg, hoff.data());
+  const int slots = sort_slots(h->sm_count, h->n_seg, h->max_nodes - 1);
+  const size_t hist = sort_hist_ints(h->seg_cap.data(), nz.data(), h->n_seg, slots, hoff.data());
   void* a = dev_alloc(h, P * 4 * 5);
-  void* b = dev_alloc(h, hist * 4);
+  void* b = dev_alloc(h, (hist + sort_tiles(hist)) * 4);
   void* c = dev_alloc(h, sizeof(int64_t) * h->n_seg);
   if (!a || !b || !c) return PIC_ENOMEM;
   h->st.z2 = (float*)a;
@@ -434,18 +438,20 @@ int sort_alloc(pic_handle* h) {
   h->st.vz2 = h->st.vy2 + P;
   h->st.id2 = (uint32_t*)(h->st.vz2 + P);
   h->st.sort_hist = (int32_t*)b;
+  h->st.sort_tsum = h->st.sort_hist + hist;
   h->st.sort_hoff = (const int64_t*)c;
   cudaError_t e = cudaMemcpyAsync(c, hoff.data(), sizeof(int64_t) * h->n_seg, cudaMemcpyHostToDevice,
                                   h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e);
-  h->sort_chunks = sort_max_chunks(h->seg_cap.data(), h->n_seg);
+  h->st.sort_slots = slots;
+  h->sort_grid = sort_grid(h->seg_cap.data(), nz.data(), h->n_seg, slots);
   h->sort_ready = true;
   drop_graph(h);
   return PIC_OK;
 }
 
-void launch_sort(pic_handle* h) { sort_launch(h->st, h->sort_chunks, h->max_nodes, h->stream); }
+void launch_sort(pic_handle* h) { sort_launch(h->st, h->sort_grid, h->max_nodes - 1, h->stream); }
 
 cudaError_t launch_field(pic_handle* h) {
   k_deposit<<<h->G, h->push_threads, h->push_smem, h->stream>>>(h->st);

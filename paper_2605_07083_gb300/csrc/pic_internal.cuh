@@ -128,7 +128,9 @@ struct DevState {
   float* E;                // [total_nodes] field of the current state (FP32 copy)
   double* phi;             // [total_nodes]
   int32_t* sort_hist;      // counting-sort histograms, per segment [cell][chunk]
+  int32_t* sort_tsum;      // sums of the histograms' tiles
   const int64_t* sort_hoff;  // [n_seg] first histogram entry of each segment
+  int sort_slots;          // blocks per wave that a segment's sort chunks are cut for
   unsigned long long* cand_buf;  // [cand_cap] null-collision candidates: (segment << 32) | absolute slot
   unsigned int* cand_count;      // [1]
   int cand_cap;
@@ -149,6 +151,8 @@ struct DevState {
   int agg;
   int kp;                  // k_mid blocks per diode for its field, per segment for its lists
 };
+
+struct SortGrid { int chunks, tiles, copies; };    // blocks per segment of the sort's kernels
 
 // Is the state after step n a profile sample?  (Sec. 3 late-time averages:
 // steps n >= window_start with (n - window_start) a multiple of the period.)

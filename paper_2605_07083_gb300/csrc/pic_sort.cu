@@ -2,173 +2,130 @@
 // segment by cell, run every few steps so that the blocks of the push kernel
 // see narrow cell ranges (short charge flushes, local shared-memory atomics).
 //
-// Four passes per sort, each a 2D grid (chunk of kSortChunk particles,
-// segment):
-//   1. per-chunk cell histogram            -> hist[g][cell][chunk]
-//   2. one block per segment: exclusive scan of hist in (cell, chunk) order
-//   3. scatter: each warp owns a contiguous sub-chunk; per-(warp, cell)
-//      offsets in shared memory; __match_any_sync ranks equal cells inside a
-//      warp, so the order of equal cells is the original order (stable)
-//   4. copy the sorted scratch arrays back
-// The cell of a particle is the fixed-point deposit's cell rule.
-#include "pic_internal.cuh"
+// The four kernels of pic_sort_core.cuh, each a 2D grid (chunk or histogram
+// tile, segment), then a copy of the sorted scratch arrays back.  The cell of
+// a particle is the fixed-point deposit's cell rule.  The grids are sized by
+// the segments' capacities, since the host does not know the live counts;
+// blocks past a segment's live particles return at once.
+#include "pic_sort_core.cuh"
 
 namespace pic {
 
-constexpr int kSortChunk = 8192;
-constexpr int kSortThreads = 256;
-constexpr int kSortWarps = kSortThreads / 32;
+using sortcore::kThreads;
+using sortcore::kTile;
+using sortcore::View;
 
-__device__ __forceinline__ int seg_nz(const DevState& st, int g) { return st.ic[g / 3].Nz; }
+constexpr int kCopyChunk = 8192;             // particles per k_sort_copy block
+// 16 warps: two blocks per SM overlap their phases, and a state sorted a few
+// steps ago has long runs in chunks of 8192 already
+constexpr int kScatWarps = 16;
 
-__device__ __forceinline__ int seg_chunks_cap(const DevState& st, int g) {
-  return (st.seg_cap[g] + kSortChunk - 1) / kSortChunk;
-}
-
-__global__ void __launch_bounds__(kSortThreads) k_sort_hist(DevState st) {
-  extern __shared__ int hs[];
-  const int g = blockIdx.y, c = blockIdx.x;
-  const int N = st.seg_count[g];
-  const int nch = (N + kSortChunk - 1) / kSortChunk;
-  if (c >= nch) return;
+// segment g of the handle; its histogram starts on a multiple of kTile
+__device__ __forceinline__ View seg_view(const DevState& st, int g) {
   const InstConst& ic = st.ic[g / 3];
-  const int Nz = ic.Nz;
-  for (int j = threadIdx.x; j < Nz; j += blockDim.x) hs[j] = 0;
-  __syncthreads();
-  const long long off = st.seg_off[g];
-  const int i0 = c * kSortChunk, i1 = min(N, i0 + kSortChunk);
-  const float inv_dz = ic.inv_dz_f;
-  for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-    int j;
-    float f;
-    cell_of(st.z[off + i], inv_dz, Nz, j, f);
-    atomicAdd(&hs[j], 1);
-  }
-  __syncthreads();
-  const int nchc = seg_chunks_cap(st, g);
-  int* h = st.sort_hist + st.sort_hoff[g];
-  for (int j = threadIdx.x; j < Nz; j += blockDim.x) h[(long long)j * nchc + c] = hs[j];
+  const long long off = st.seg_off[g], hoff = st.sort_hoff[g];
+  View v;
+  v.z = st.z + off; v.vx = st.vx + off; v.vy = st.vy + off; v.vz = st.vz + off; v.id = st.id + off;
+  v.zo = st.z2 + off; v.vxo = st.vx2 + off; v.vyo = st.vy2 + off; v.vzo = st.vz2 + off;
+  v.ido = st.id2 + off;
+  v.hist = st.sort_hist + hoff;
+  v.tsum = st.sort_tsum + hoff / kTile;
+  v.n = st.seg_count[g];
+  v.chunk = sortcore::chunk_of(v.n, kScatWarps, st.sort_slots);
+  v.nch = (v.n + v.chunk - 1) / v.chunk;
+  v.Nz = ic.Nz;
+  v.inv_dz = ic.inv_dz_f;
+  return v;
 }
 
-__global__ void __launch_bounds__(1024) k_sort_scan(DevState st) {
+__global__ void __launch_bounds__(kThreads) k_sort_hist(DevState st) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const View v = seg_view(st, blockIdx.y);
+  if ((int)blockIdx.x >= v.nch) return;
+  sortcore::sort_hist(v, blockIdx.x, reinterpret_cast<int*>(smem));
+}
+
+__global__ void __launch_bounds__(kThreads) k_sort_tilesum(DevState st) {
   __shared__ int ws[32];
-  const int g = blockIdx.x;
-  const int N = st.seg_count[g];
-  const int nch = (N + kSortChunk - 1) / kSortChunk;
-  if (nch == 0) return;
-  const int nchc = seg_chunks_cap(st, g);
-  const int Nz = seg_nz(st, g);
-  int* h = st.sort_hist + st.sort_hoff[g];
-  // entries (cell j, chunk c < nch) in cell-major order; chunks >= nch are unused
-  const long long n = (long long)Nz * nch;
-  int carry = 0;
-  for (long long base = 0; base < n; base += blockDim.x) {
-    const long long k = base + threadIdx.x;
-    int v = 0;
-    long long addr = 0;
-    if (k < n) {
-      const long long j = k / nch, c = k - j * nch;
-      addr = j * nchc + c;
-      v = h[addr];
-    }
-    int tot;
-    const int ex = block_exclusive_scan<int>(v, &tot, ws);
-    if (k < n) h[addr] = carry + ex;
-    carry += tot;
-  }
+  const View v = seg_view(st, blockIdx.y);
+  if ((int)blockIdx.x >= sortcore::tile_count(v)) return;
+  sortcore::sort_tilesum(v, blockIdx.x, ws);
 }
 
-__global__ void __launch_bounds__(kSortThreads) k_sort_scatter(DevState st) {
-  extern __shared__ int woff[];               // [kSortWarps][Nz]
-  const int g = blockIdx.y, c = blockIdx.x;
+__global__ void __launch_bounds__(kThreads) k_sort_scan(DevState st) {
+  __shared__ int ws[32];
+  const View v = seg_view(st, blockIdx.y);
+  if ((int)blockIdx.x >= sortcore::tile_count(v)) return;
+  sortcore::sort_scan(v, blockIdx.x, ws);
+}
+
+__global__ void __launch_bounds__(32 * kScatWarps, 2) k_sort_scatter(DevState st) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int ws[32];
+  const View v = seg_view(st, blockIdx.y);
+  if ((int)blockIdx.x >= v.nch) return;
+  sortcore::sort_scatter<kScatWarps>(v, blockIdx.x, smem, ws);
+}
+
+// The sorted particles back into the handle's arrays, four slots per access:
+// segments start on a multiple of 32 slots and hold a multiple of 32, so the
+// last access of a segment stays inside it (its slots past the live ones
+// hold nothing).
+__global__ void __launch_bounds__(kThreads) k_sort_copy(DevState st) {
+  const int g = blockIdx.y;
   const int N = st.seg_count[g];
-  const int nch = (N + kSortChunk - 1) / kSortChunk;
-  if (c >= nch) return;
-  const InstConst& ic = st.ic[g / 3];
-  const int Nz = ic.Nz;
-  const float inv_dz = ic.inv_dz_f;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int q0 = blockIdx.x * (kCopyChunk / 4), q1 = min((N + 3) >> 2, q0 + kCopyChunk / 4);
   const long long off = st.seg_off[g];
-  const int i0 = c * kSortChunk, i1 = min(N, i0 + kSortChunk);
-  const int per = (kSortChunk / kSortWarps);
-  const int w0 = i0 + warp * per, w1 = min(i1, w0 + per);
-  for (int k = threadIdx.x; k < kSortWarps * Nz; k += blockDim.x) woff[k] = 0;
-  __syncthreads();
-  int* my = woff + warp * Nz;
-  for (int i = w0 + lane; i < w1; i += 32) {
-    int j;
-    float f;
-    cell_of(st.z[off + i], inv_dz, Nz, j, f);
-    atomicAdd(&my[j], 1);
-  }
-  __syncthreads();
-  const int nchc = seg_chunks_cap(st, g);
-  const int* h = st.sort_hist + st.sort_hoff[g];
-  for (int j = threadIdx.x; j < Nz; j += blockDim.x) {
-    int run = h[(long long)j * nchc + c];
-    for (int w = 0; w < kSortWarps; ++w) {
-      const int cnt = woff[w * Nz + j];
-      woff[w * Nz + j] = run;
-      run += cnt;
-    }
-  }
-  __syncthreads();
-  const unsigned lt = (1u << lane) - 1u;
-  for (int base = w0; base < w1; base += 32) {
-    const int i = base + lane;
-    const bool act = i < w1;
-    const unsigned am = __ballot_sync(0xffffffffu, act);
-    int j = -1;
-    if (act) {
-      float f;
-      cell_of(st.z[off + i], inv_dz, Nz, j, f);
-    }
-    const unsigned peers = __match_any_sync(0xffffffffu, j) & am;
-    int pos = 0;
-    if (act) pos = my[j] + __popc(peers & lt);
-    __syncwarp();
-    if (act && (peers & lt) == 0u) my[j] += __popc(peers);
-    __syncwarp();
-    if (act) {
-      st.z2[off + pos] = st.z[off + i];
-      st.vx2[off + pos] = st.vx[off + i];
-      st.vy2[off + pos] = st.vy[off + i];
-      st.vz2[off + pos] = st.vz[off + i];
-      st.id2[off + pos] = st.id[off + i];
-    }
+  const float* from[4] = {st.z2 + off, st.vx2 + off, st.vy2 + off, st.vz2 + off};
+  float* to[4] = {st.z + off, st.vx + off, st.vy + off, st.vz + off};
+  const uint4* ifrom = reinterpret_cast<const uint4*>(st.id2 + off);
+  uint4* ito = reinterpret_cast<uint4*>(st.id + off);
+  for (int q = q0 + threadIdx.x; q < q1; q += kThreads) {
+    float4 x[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = reinterpret_cast<const float4*>(from[k])[q];
+    const uint4 i = ifrom[q];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) reinterpret_cast<float4*>(to[k])[q] = x[k];
+    ito[q] = i;
   }
 }
 
-__global__ void __launch_bounds__(kSortThreads) k_sort_copy(DevState st) {
-  const int g = blockIdx.y, c = blockIdx.x;
-  const int N = st.seg_count[g];
-  const int i0 = c * kSortChunk, i1 = min(N, i0 + kSortChunk);
-  const long long off = st.seg_off[g];
-  for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-    st.z[off + i] = st.z2[off + i];
-    st.vx[off + i] = st.vx2[off + i];
-    st.vy[off + i] = st.vy2[off + i];
-    st.vz[off + i] = st.vz2[off + i];
-    st.id[off + i] = st.id2[off + i];
-  }
+// Blocks per wave that a segment's chunks are cut for: the segments share the
+// chip, with two blocks per SM where the counters of two fit
+int sort_slots(int sms, int n_seg, int max_nz) {
+  const int per_sm = sortcore::scatter_smem(max_nz, kScatWarps) <= 110 * 1024 ? 2 : 1;
+  return max(1, per_sm * sms / n_seg);
 }
 
-size_t sort_hist_ints(const int32_t* seg_cap, const int* seg_nz, int n_seg, int64_t* hoff) {
+static long long seg_hist_ints(int cap, int nz, int slots) {
+  return (long long)nz * sortcore::max_columns(cap, kScatWarps, slots);
+}
+
+// histogram entries of all segments (each segment's a multiple of kTile)
+size_t sort_hist_ints(const int32_t* seg_cap, const int* seg_nz, int n_seg, int slots,
+                      int64_t* hoff) {
   size_t tot = 0;
   for (int g = 0; g < n_seg; ++g) {
     hoff[g] = (int64_t)tot;
-    tot += (size_t)seg_nz[g] * (size_t)((seg_cap[g] + kSortChunk - 1) / kSortChunk);
+    tot += (size_t)(seg_hist_ints(seg_cap[g], seg_nz[g], slots) + kTile - 1) / kTile * kTile;
   }
   return tot;
 }
 
-int sort_max_chunks(const int32_t* seg_cap, int n_seg) {
-  int m = 1;
-  for (int g = 0; g < n_seg; ++g) m = max(m, (seg_cap[g] + kSortChunk - 1) / kSortChunk);
-  return m;
-}
+size_t sort_tiles(size_t hist_ints) { return hist_ints / kTile; }
 
-size_t sort_scatter_smem(int max_nz) { return (size_t)kSortWarps * max_nz * sizeof(int); }
+// grid sizes: chunks, histogram tiles and copy blocks of the largest segment
+SortGrid sort_grid(const int32_t* seg_cap, const int* seg_nz, int n_seg, int slots) {
+  SortGrid r{1, 1, 1};
+  for (int g = 0; g < n_seg; ++g) {
+    const long long e = seg_hist_ints(seg_cap[g], seg_nz[g], slots);
+    r.chunks = max(r.chunks, sortcore::max_columns(seg_cap[g], kScatWarps, slots));
+    r.tiles = max(r.tiles, (int)((e + kTile - 1) / kTile));
+    r.copies = max(r.copies, (seg_cap[g] + kCopyChunk - 1) / kCopyChunk);
+  }
+  return r;
+}
 
 // raise the kernels' dynamic shared-memory limit to the opt-in maximum less
 // their static shared memory
@@ -185,12 +142,13 @@ cudaError_t sort_prepare(int optin) {
   return cudaSuccess;
 }
 
-void sort_launch(const DevState& st, int max_chunks, int max_nz, cudaStream_t s) {
-  const dim3 grid(max_chunks, st.n_seg);
-  k_sort_hist<<<grid, kSortThreads, max_nz * sizeof(int), s>>>(st);
-  k_sort_scan<<<st.n_seg, 1024, 0, s>>>(st);
-  k_sort_scatter<<<grid, kSortThreads, sort_scatter_smem(max_nz), s>>>(st);
-  k_sort_copy<<<grid, kSortThreads, 0, s>>>(st);
+void sort_launch(const DevState& st, const SortGrid& r, int max_nz, cudaStream_t s) {
+  const dim3 chunks(r.chunks, st.n_seg), tiles(r.tiles, st.n_seg), copies(r.copies, st.n_seg);
+  k_sort_hist<<<chunks, kThreads, max_nz * sizeof(int), s>>>(st);
+  k_sort_tilesum<<<tiles, kThreads, 0, s>>>(st);
+  k_sort_scan<<<tiles, kThreads, 0, s>>>(st);
+  k_sort_scatter<<<chunks, 32 * kScatWarps, sortcore::scatter_smem(max_nz, kScatWarps), s>>>(st);
+  k_sort_copy<<<copies, kThreads, 0, s>>>(st);
 }
 
 }  // namespace pic
