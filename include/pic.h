@@ -113,7 +113,8 @@ typedef struct pic_tuning {
     int32_t push_threads;     /* threads per block of the particle kernels (64..384, multiple of
                                  32; default: the size that keeps closest to 24 resident warps
                                  per SM for the handle's cell count, the first of 384, 256,
-                                 128, 160, ... that does) */
+                                 128, 160, ... that does, or one block of 640..768 threads
+                                 per SM where the cell grid leaves two blocks too few) */
     int32_t push_blocks_per_sm;  /* cap on resident blocks per SM (default: occupancy limit) */
     int32_t sort_period;      /* counting sort by cell every this many steps; < 0 disables */
     int32_t graph_steps;      /* longest step loop captured as one CUDA graph (default 64,
@@ -334,8 +335,9 @@ const char* pic_last_error(const pic_handle* h);
  * application, a plugin inside another framework's memory pool), where a
  * cudaMalloc could fail, block or synchronise the device at the wrong time.
  * The caller passes inputs and outputs; the scratch (a (cell, chunk)
- * histogram and its tile sums) is a fixed 4 MiB device array (and 1 KiB) inside this library that every
- * GPU loading the library holds until the process exits.
+ * histogram and its tile sums) is a fixed 4 MiB and 1 KiB of device memory
+ * inside this library that every GPU loading the library holds until the
+ * process exits.
  *
  * z..id: n input particles (device); z_out..id_out: n outputs (device), not
  * aliasing the inputs.  Output = input stably sorted by the fixed-point cell

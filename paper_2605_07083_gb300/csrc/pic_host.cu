@@ -18,8 +18,13 @@
 namespace pic {
 __global__ void k_push(DevState st);
 __global__ void k_push32(DevState st);
+__global__ void k_push_wide(DevState st);
+__global__ void k_push_many(DevState st);
+__global__ void k_push32_many(DevState st);
+__global__ void k_push_wide_many(DevState st);
 __global__ void k_deposit(DevState st);
 __global__ void k_mid(DevState st);
+__global__ void k_mid_many(DevState st);
 __global__ void k_post(DevState st);
 __global__ void k_field(DevState st);
 __global__ void k_profile(DevState st);
@@ -265,10 +270,12 @@ cudaError_t raise_smem_limits(int device) {
   int optin = 0;
   cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   if (e != cudaSuccess) return e;
-  const void* fns[] = {(const void*)k_push, (const void*)k_push32,
+  const void* fns[] = {(const void*)k_push, (const void*)k_push32, (const void*)k_push_wide,
+                       (const void*)k_push_many, (const void*)k_push32_many,
+                       (const void*)k_push_wide_many,
                        (const void*)k_deposit, (const void*)k_field,
                        (const void*)k_post, (const void*)k_profile, (const void*)k_phi,
-                       (const void*)k_mid};
+                       (const void*)k_mid, (const void*)k_mid_many};
   for (const void* f : fns) {
     e = set_dynamic_smem_limit(f, optin);
 
@@ -287,12 +294,19 @@ size_t push_smem_bytes(const pic_handle* h, int threads, int chunk) {
 }
 
 using PushKernel = void (*)(DevState);
-PushKernel push_kernel(int chunk) { return chunk == 32 ? k_push32 : k_push; }
+constexpr int kPushThreads = 384;            // most threads of a block that shares its SM
+PushKernel push_kernel(const pic_handle* h, int threads, int chunk) {
+  if (h->st.cand_many)
+    return threads > kPushThreads ? k_push_wide_many : chunk == 32 ? k_push32_many : k_push_many;
+  return threads > kPushThreads ? k_push_wide : chunk == 32 ? k_push32 : k_push;
+}
+
+PushKernel mid_kernel(const pic_handle* h) { return h->st.cand_many ? k_mid_many : k_mid; }
 
 // resident warps per SM of a push shape (0 if it does not fit)
 int push_warps(const pic_handle* h, int threads, int chunk) {
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_kernel(chunk), threads,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_kernel(h, threads, chunk), threads,
                                                     push_smem_bytes(h, threads, chunk)) !=
       cudaSuccess)
     return 0;
@@ -304,19 +318,28 @@ int push_warps(const pic_handle* h, int threads, int chunk) {
 // slots, fewer leave dependency waits exposed).  The shared-memory footprint
 // grows with the cell count and the chunk, so pick the block size and chunk
 // that get closest to 24 warps from below, preferring 64-quad chunks, then
-// 384 threads (two blocks per SM), on ties.  A caller's choice of either is
-// kept.
+// 384 threads (two blocks per SM), on ties.  Where two blocks with 64-quad
+// chunks leave fewer than 20 warps (from ~2900 cells), one block of up to 24
+// warps, which holds the grid once, is tried before 32-quad chunks: 704
+// threads against 2 x 320 at 4096 cells, push 112 -> 107 us on the paper
+// scan.  With room for two blocks it is the slower one (64-diode sweep, 22
+// warps in two blocks against 24 in one: 166 and 170 us; production diode 44
+// and 45: all of a block's warps wait for its slowest).  A caller's choice of
+// either is kept.
 void default_push_shape(pic_handle* h) {
   int best_t = h->threads_set ? h->push_threads : 384;
   int best_c = h->chunk_set ? h->push_chunk : 64;
   int best_w = -1;
+  const auto consider = [&](int t, int c) {
+    if (h->chunk_set && c != h->push_chunk) return;
+    if (h->threads_set && t != h->push_threads) return;
+    const int w = std::min(push_warps(h, t, c), 24);
+    if (w > best_w) { best_t = t; best_c = c; best_w = w; }
+  };
   for (int c : {64, 32}) {
-    if (h->chunk_set && c != h->push_chunk) continue;
-    for (int t : {384, 256, 128, 160, 192, 224, 288, 320, 352}) {
-      if (h->threads_set && t != h->push_threads) continue;
-      const int w = std::min(push_warps(h, t, c), 24);
-      if (w > best_w) { best_t = t; best_c = c; best_w = w; }
-    }
+    for (int t : {384, 256, 128, 160, 192, 224, 288, 320, 352}) consider(t, c);
+    if (c == 64 && best_w < 20)
+      for (int t : {768, 736, 704, 672, 640}) consider(t, c);
   }
   h->push_threads = best_t;
   h->push_chunk = best_c;
@@ -325,12 +348,22 @@ void default_push_shape(pic_handle* h) {
 int set_launch_shape(pic_handle* h) {
   cudaError_t e = raise_smem_limits(h->device);
   if (e != cudaSuccess) return cuda_fail(h, e);
+  // many candidates: more expected per step (probability x capacity) than one
+  // per thread of one k_mid block per SM.  Then the push writes records that
+  // spare k_mid three random reads each (paper scan, 1 % candidates: k_mid 29
+  // -> 22 us for 2 us more of the push); with few the records only cost the
+  // push registers (64-diode sweep: push 166 -> 171 us).
+  double cand = 0.0;
+  for (int i = 0; i < h->n_inst; ++i)
+    for (int s = 0; s < 3; ++s)
+      cand += (double)h->ic[i].t_cand[s] * (1.0 / 4294967296.0) * (double)h->seg_cap[3 * i + s];
+  h->st.cand_many = cand > (double)h->sm_count * kPostThreads ? 1 : 0;
   default_push_shape(h);
   h->push_smem = push_smem_bytes(h, h->push_threads, h->push_chunk);
   h->field_smem = (size_t)h->max_nodes * 8;
   int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_kernel(h->push_chunk),
-                                                    h->push_threads, h->push_smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &occ, push_kernel(h, h->push_threads, h->push_chunk), h->push_threads, h->push_smem);
   if (e != cudaSuccess) return cuda_fail(h, e);
   if (occ < 1) occ = 1;
   const int per_sm = h->blocks_per_sm > 0 ? std::min(h->blocks_per_sm, occ) : occ;
@@ -342,15 +375,12 @@ int set_launch_shape(pic_handle* h) {
   // blocks each when the diodes are few (their FP64 work then shares no SM)
   h->st.kp = std::max(1, std::min(kMaxParts, h->sm_count / (4 * h->n_inst)));
   h->st.W = h->push_threads / 32;
-  // collision blocks of k_mid: one per SM, two where the expected candidates
-  // per step (candidate probability x capacity) would give every thread of
-  // one block per SM more than one collision (measured: 1.2x faster k_mid at
-  // ~1 % candidates of 22M particles, 0.9x at 0.01 % of 10M)
-  double cand = 0.0;
-  for (int i = 0; i < h->n_inst; ++i)
-    for (int s = 0; s < 3; ++s)
-      cand += (double)h->ic[i].t_cand[s] * (1.0 / 4294967296.0) * (double)h->seg_cap[3 * i + s];
-  h->mcc_blocks = cand > (double)h->sm_count * kPostThreads ? 2 * h->sm_count : h->sm_count;
+  // collision blocks of k_mid: one per SM; with many candidates all the
+  // places its other blocks leave free, so that they are all resident at once
+  // (two blocks per SM: a second wave would start when the first blocks end,
+  // ~10 us later on the paper scan)
+  const int places = 2 * h->sm_count - 4 * h->n_inst * h->st.kp - 1;
+  h->mcc_blocks = h->st.cand_many ? std::max(h->sm_count, places) : h->sm_count;
   const size_t need = (size_t)h->n_seg * h->G;
   if (need > h->dcount_ints) {
     void* p = dev_alloc(h, need * sizeof(int32_t));
@@ -404,6 +434,9 @@ int set_launch_shape(pic_handle* h) {
   // k_mid: a diode's charge and emission histogram, or a segment's piece
   // ranges and prefix; k_post: the staged absorbed list or the event keys
   h->mid_smem = std::max((size_t)h->max_nodes * 20, (size_t)(h->G + 1) * 12) + 16;
+  // or the collision blocks' constants, steps and tallies
+  if (h->n_inst <= kSmemInst)
+    h->mid_smem = std::max(h->mid_smem, h->n_inst * (sizeof(InstConst) + 8 + 4 * kTallies));
   h->post_smem = std::max((size_t)kDeadSmem * 4, (size_t)kEvCap * 8) + 16;
   // profile sampler: blocks per segment so that none bins more than
   // kHistMaxParticles particles (its 32-bit counters), else about two blocks
@@ -485,8 +518,8 @@ void launch_profile(pic_handle* h) {
 
 // one time step; the sort, when due, follows the step
 cudaError_t launch_step(pic_handle* h) {
-  push_kernel(h->push_chunk)<<<h->G, h->push_threads, h->push_smem, h->stream>>>(h->st);
-  k_mid<<<mid_blocks(h), kPostThreads, h->mid_smem, h->stream>>>(h->st);
+  push_kernel(h, h->push_threads, h->push_chunk)<<<h->G, h->push_threads, h->push_smem, h->stream>>>(h->st);
+  mid_kernel(h)<<<mid_blocks(h), kPostThreads, h->mid_smem, h->stream>>>(h->st);
   k_post<<<3 * h->n_inst, kPostThreads, h->post_smem, h->stream>>>(h->st);
   launch_profile(h);
   h->host_step += 1;
@@ -503,8 +536,8 @@ int build_graph(pic_handle* h, int len, cudaGraphExec_t* out) {
   cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaStreamBeginCapture");
   for (int i = 0; i < len; ++i) {
-    push_kernel(h->push_chunk)<<<h->G, h->push_threads, h->push_smem, h->stream>>>(h->st);
-    k_mid<<<mid_blocks(h), kPostThreads, h->mid_smem, h->stream>>>(h->st);
+    push_kernel(h, h->push_threads, h->push_chunk)<<<h->G, h->push_threads, h->push_smem, h->stream>>>(h->st);
+    mid_kernel(h)<<<mid_blocks(h), kPostThreads, h->mid_smem, h->stream>>>(h->st);
     k_post<<<3 * h->n_inst, kPostThreads, h->post_smem, h->stream>>>(h->st);
     launch_profile(h);
     if (sort_due(h, i + 1)) launch_sort(h);
@@ -708,7 +741,7 @@ int pic_create(const pic_config* cfgs, int n_instances, void* cuda_stream,
   p[13] = dev_alloc(h, sizeof(InstDyn) * h->n_inst);
   // candidates per step: far above the expected P_cand * N (<= 1e-2 of all slots)
   const int64_t cand_cap = std::min<int64_t>(h->total_cap / 16 + 65536, 1LL << 30);
-  p[14] = dev_alloc(h, sizeof(unsigned long long) * (size_t)cand_cap + 256);
+  p[14] = dev_alloc(h, (sizeof(uint4) + sizeof(uint32_t)) * (size_t)cand_cap + 256);
   p[15] = dev_alloc(h, sizeof(PostScratch) * h->n_inst);
   for (int k = 0; k < 16; ++k)
     if (!p[k]) { pic_destroy(h); return PIC_ENOMEM; }
@@ -728,8 +761,9 @@ int pic_create(const pic_config* cfgs, int n_instances, void* cuda_stream,
   st.ic = (const InstConst*)p[12];
   st.dyn = (InstDyn*)p[13];
   st.cand_cap = (int)cand_cap;
-  st.cand_buf = (unsigned long long*)p[14];
-  st.cand_count = (unsigned int*)((char*)p[14] + sizeof(unsigned long long) * (size_t)cand_cap);
+  st.cand_rec = (uint4*)p[14];
+  st.cand_seg = (uint32_t*)(st.cand_rec + cand_cap);
+  st.cand_count = (unsigned int*)(st.cand_seg + cand_cap);
   st.post = (PostScratch*)p[15];
   // counting-sort scratch: a second particle set plus histograms
   st.z2 = nullptr;
@@ -905,9 +939,9 @@ int pic_profile_steps(pic_handle* h, int64_t n_steps, pic_profile* out) {
   for (int64_t i = 0; i < n_steps; ++i) {
     cudaEvent_t* e = &ev[6 * i];
     cudaEventRecord(e[0], h->stream);
-    push_kernel(h->push_chunk)<<<h->G, h->push_threads, h->push_smem, h->stream>>>(h->st);
+    push_kernel(h, h->push_threads, h->push_chunk)<<<h->G, h->push_threads, h->push_smem, h->stream>>>(h->st);
     cudaEventRecord(e[1], h->stream);
-    k_mid<<<mid_blocks(h), kPostThreads, h->mid_smem, h->stream>>>(h->st);
+    mid_kernel(h)<<<mid_blocks(h), kPostThreads, h->mid_smem, h->stream>>>(h->st);
     cudaEventRecord(e[5], h->stream);
     k_post<<<3 * h->n_inst, kPostThreads, h->post_smem, h->stream>>>(h->st);
     launch_profile(h);

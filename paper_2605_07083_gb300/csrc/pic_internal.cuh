@@ -11,6 +11,8 @@ constexpr int kMaxNz = 4096;          // shared-memory grid limit (nodes = Nz + 
 constexpr int kMaxInstances = 1024;
 constexpr int kEvCap = 2048;          // ionisation events per instance per step
 constexpr int kPostThreads = 512;
+constexpr int kSmemInst = 64;         // most diodes whose constants k_mid's collisions keep in smem
+constexpr int kTallies = 9;           // window tallies: outcomes 0..5, candidates of species 0..2
 constexpr int kMaxParts = 4;          // k_mid blocks per diode field / per segment list
 constexpr int kHistMaxParticles = (1 << 20) - 256;
 // push-block weights (shares of the particle range): nominal, bounds
@@ -67,6 +69,8 @@ struct InstConst {
   double m_d[3];
   int64_t window_start;
 };
+
+static_assert(sizeof(InstConst) % 8 == 0, "copied as words, followed by 64-bit words");
 
 // Mutable per-instance state.
 struct InstDyn {
@@ -131,7 +135,12 @@ struct DevState {
   int32_t* sort_tsum;      // sums of the histograms' tiles
   const int64_t* sort_hoff;  // [n_seg] first histogram entry of each segment
   int sort_slots;          // blocks per wave that a segment's sort chunks are cut for
-  unsigned long long* cand_buf;  // [cand_cap] null-collision candidates: (segment << 32) | absolute slot
+  // null-collision candidates, [cand_cap]: with cand_many the absolute slot, the id and the
+  // bits of z and v_z after the push, and the segment in cand_seg; else one 64-bit word each
+  // in the same buffer, (segment << 32) | absolute slot
+  uint4* cand_rec;
+  uint32_t* cand_seg;
+  int cand_many;           // 1: many candidates are expected per step
   unsigned int* cand_count;      // [1]
   int cand_cap;
   const InstConst* ic;

@@ -193,12 +193,11 @@ __device__ __forceinline__ void deposit_quad(const Hist& h, const float4& z4, fl
 // cumulative n sigma_k(E_rel) |g| (null beyond), words 2-3 the isotropic
 // direction.  Block 1: neutral partner velocity (Maxwellian at T_n).  Block
 // 2: ionisation energy split and the ejected electron's direction.
-// Returns the new v_z; writes v_x, v_y in place.  Rare path: kept out of line.
-__device__ __forceinline__ float collide(const InstConst* __restrict__ icg, InstDyn* dyn,
-                                      Event* evb, float* vxp, float* vyp, int sp, uint32_t pid,
-                                      uint32_t stepw, long long step, float z, float vz,
-                                      int& code_out) {
-  const InstConst& ic = *icg;
+// Velocities are changed in place; returns the outcome (0: null).
+__device__ __forceinline__ int collide(const InstConst& ic, InstDyn* dyn, Event* evb, int sp,
+                                       uint32_t pid, long long step, float z, float& vx, float& vy,
+                                       float& vz) {
+  const uint32_t stepw = (uint32_t)step;
   const uint32_t k0 = ic.key0[sp], k1 = ic.key1;
   const uint4 A = philox10(make_uint4(pid, stepw, 0u, TAG_MCC), k0, k1);
   const uint4 B = philox10(make_uint4(pid, stepw, 1u, TAG_MCC), k0, k1);
@@ -207,7 +206,6 @@ __device__ __forceinline__ float collide(const InstConst* __restrict__ icg, Inst
   box_muller(B.z, B.w, n2, n3);
   const float sn = ic.sig_n[sp];
   const float vnx = sn * n0, vny = sn * n1, vnz = sn * n2;
-  const float vx = *vxp, vy = *vyp;
   const float gx = vx - vnx, gy = vy - vny, gz = vz - vnz;
   const float g2 = gx * gx + gy * gy + gz * gz;
   const float gm = sqrtf(g2);
@@ -287,40 +285,40 @@ __device__ __forceinline__ float collide(const InstConst* __restrict__ icg, Inst
       nvz = fm * vz + fM * vnz + fM * gm * dz;
     }
   }
-  code_out = code;
-  if (code != 0) {
-    *vxp = nvx;
-    *vyp = nvy;
-  }
-  return nvz;
+  vx = nvx;
+  vy = nvy;
+  vz = nvz;
+  return code;
 }
 
 // The collisions of the step's null-collision candidates: thread t of a
-// stride-`stride` team takes candidates t, t + stride, ...  A record is
-// (segment << 32) | absolute slot; the thread's first record is read in the
-// round trip of the count (a record at or past the count is never used, and
-// the buffer holds cand_cap of them), so a candidate's particle is two round
-// trips from the kernel's start.
-__device__ void mcc_candidates(const DevState& st, unsigned t, unsigned stride) {
+// stride-`stride` team takes candidates t, t + stride, ...  A record is read
+// in the round trip of the count (one at or past the count is never used, and
+// the buffer holds cand_cap of them).
+
+// Few candidates (well under one per thread): the chain record -> particle ->
+// collision is all there is, so nothing is staged.  A warp adds its window
+// tallies per (segment, outcome).
+__device__ void mcc_few(const DevState& st, unsigned t, unsigned stride) {
   const unsigned cap = (unsigned)st.cand_cap;
-  const unsigned long long e_first = t < cap ? st.cand_buf[t] : 0ull;
+  const unsigned long long* rec = reinterpret_cast<const unsigned long long*>(st.cand_rec);
+  const unsigned long long e_first = t < cap ? rec[t] : 0ull;
   const unsigned n = min(*st.cand_count, cap);
   for (unsigned k = t; k < n; k += stride) {
-    const unsigned long long e = k == t ? e_first : st.cand_buf[k];
+    const unsigned long long e = k == t ? e_first : rec[k];
     const int g = (int)(e >> 32);
     const long long slot = (long long)(e & 0xffffffffu);
     const int inst = g / 3, sp = g - 3 * inst;
     const long long step = st.dyn[inst].step;
-    int code;
-    const float vz = collide(st.ic + inst, st.dyn + inst, st.ev_buf + (long long)inst * kEvCap,
-                             st.vx + slot, st.vy + slot, sp, st.id[slot], (uint32_t)step, step,
-                             st.z[slot], st.vz[slot], code);
-    st.vz[slot] = vz;
+    float vx = st.vx[slot], vy = st.vy[slot], vz = st.vz[slot];
+    const int code = collide(st.ic[inst], st.dyn + inst, st.ev_buf + (long long)inst * kEvCap, sp,
+                             st.id[slot], step, st.z[slot], vx, vy, vz);
+    if (code != 0) {
+      st.vx[slot] = vx;
+      st.vy[slot] = vy;
+      st.vz[slot] = vz;
+    }
     if (step >= st.ic[inst].window_start) {
-      // window tallies of candidates and outcomes: lanes with the same
-      // (segment, outcome) add once -- one 64-bit atomic per candidate on a
-      // handful of per-diode counters would serialise when candidates are
-      // many (about 1 % of the particles per step at 40 V)
       const unsigned mask = __activemask();
       const unsigned peers = __match_any_sync(mask, ((unsigned)g << 3) | (unsigned)code);
       if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) {
@@ -328,6 +326,102 @@ __device__ void mcc_candidates(const DevState& st, unsigned t, unsigned stride) 
         atomicAdd(&st.dyn[inst].cand[sp], c);
         atomicAdd(&st.dyn[inst].coll[code], c);
       }
+    }
+  }
+}
+
+// Many candidates (DevState::cand_many).  What bounds it: v_x and v_y come
+// from random sectors of HBM and the velocities go back to them; with only
+// the slot in a record the five reads per candidate took 10 of k_mid's 24 us
+// on the 11-diode paper scan (108k candidates a step).  A record therefore
+// holds the rest of the particle as the push left it, and the next
+// candidate's v_x and v_y are in flight while one collides.  Up to kSmemInst
+// diodes the constants, the step and the window tallies lie in shared memory:
+// a warp's candidates come from all over the list, so adding per warp left
+// ~20 adds per warp on a few dozen 64-bit counters, which the L2 serialises.
+// k_mid there: 31.1 -> 21.9 us (event-timed; 27.7 with the tallies alone).
+__device__ void mcc_many(const DevState& st, unsigned t, unsigned stride, unsigned char* smem) {
+  const unsigned cap = (unsigned)st.cand_cap, t1 = t + stride;
+  uint4 r = make_uint4(0u, 0u, 0u, 0u), r_next = r;
+  unsigned g = 0u, g_next = 0u;
+  if (t < cap) {
+    r = st.cand_rec[t];
+    g = st.cand_seg[t];
+  }
+  if (t1 < cap) {
+    r_next = st.cand_rec[t1];
+    g_next = st.cand_seg[t1];
+  }
+  const unsigned n = min(*st.cand_count, cap);
+  if (__syncthreads_or(t < n) == 0) return;             // nothing for this block
+  float vx = 0.0f, vy = 0.0f;
+  if (t < n) {
+    vx = st.vx[r.x];
+    vy = st.vy[r.x];
+  }
+  const bool in_smem = st.n_inst <= kSmemInst;
+  InstConst* ics = reinterpret_cast<InstConst*>(smem);
+  long long* steps = reinterpret_cast<long long*>(ics + (in_smem ? st.n_inst : 0));
+  unsigned* tally = reinterpret_cast<unsigned*>(steps + (in_smem ? st.n_inst : 0));
+  if (in_smem) {
+    const int words = st.n_inst * (int)(sizeof(InstConst) / 4);
+    const int* src = reinterpret_cast<const int*>(st.ic);
+    for (int w = threadIdx.x; w < words; w += blockDim.x) reinterpret_cast<int*>(ics)[w] = src[w];
+    for (int i = threadIdx.x; i < st.n_inst; i += blockDim.x) steps[i] = st.dyn[i].step;
+    for (int i = threadIdx.x; i < kTallies * st.n_inst; i += blockDim.x) tally[i] = 0u;
+    __syncthreads();
+  }
+  for (unsigned k = t; k < n; k += stride) {
+    float vx_next = 0.0f, vy_next = 0.0f;
+    const uint4 c = r;
+    const int inst = (int)g / 3, sp = (int)g - 3 * inst;
+    const unsigned seg = g;
+    if (k + stride < n) {
+      vx_next = st.vx[r_next.x];
+      vy_next = st.vy[r_next.x];
+      r = r_next;
+      g = g_next;
+      const unsigned k2 = k + 2u * stride;
+      if (k2 < n) {
+        r_next = st.cand_rec[k2];
+        g_next = st.cand_seg[k2];
+      }
+    }
+    const InstConst& ic = in_smem ? ics[inst] : st.ic[inst];
+    const long long step = in_smem ? steps[inst] : st.dyn[inst].step;
+    float vz = __uint_as_float(c.w);
+    const int code = collide(ic, st.dyn + inst, st.ev_buf + (long long)inst * kEvCap, sp, c.y,
+                             step, __uint_as_float(c.z), vx, vy, vz);
+    if (code != 0) {
+      st.vx[c.x] = vx;
+      st.vy[c.x] = vy;
+      st.vz[c.x] = vz;
+    }
+    if (step >= ic.window_start) {
+      if (in_smem) {
+        atomicAdd(&tally[kTallies * inst + code], 1u);
+        atomicAdd(&tally[kTallies * inst + 6 + sp], 1u);
+      } else {
+        const unsigned mask = __activemask();
+        const unsigned peers = __match_any_sync(mask, (seg << 3) | (unsigned)code);
+        if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) {
+          const unsigned long long cnt = (unsigned long long)__popc(peers);
+          atomicAdd(&st.dyn[inst].cand[sp], cnt);
+          atomicAdd(&st.dyn[inst].coll[code], cnt);
+        }
+      }
+    }
+    vx = vx_next;
+    vy = vy_next;
+  }
+  if (in_smem) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < kTallies * st.n_inst; i += blockDim.x) {
+      const unsigned cnt = tally[i];
+      if (cnt == 0u) continue;
+      InstDyn* d = st.dyn + i / kTallies;
+      const int w = i % kTallies;
+      atomicAdd(w < 6 ? &d->coll[w] : &d->cand[w - 6], (unsigned long long)cnt);
     }
   }
 }
@@ -525,10 +619,15 @@ __device__ __forceinline__ bool stage_ready(const DevState& st, unsigned long lo
 
 // Collision candidates -> the compact global list (one atomic per warp);
 // absorbed slots -> this warp's ordered list (warp scans).  Called by all 32
-// lanes for a chunk in which some lane has either; q is the lane's quad.
+// lanes for a chunk in which some lane has either; q is the lane's quad and
+// z, v, id its particles after the push.  kMany: a candidate's record carries
+// them, so that k_mid, which meets the candidates in a random order, fetches
+// only v_x and v_y from the particle arrays.
+template <bool kMany>
 __device__ __forceinline__ void record_events(const DevState& st, int g, int inst, long long off,
-                                              int q, unsigned cm, unsigned dm, uint32_t* dbuf,
-                                              int& dead_run, int lane) {
+                                              int q, unsigned cm, unsigned dm, const float (&z)[4],
+                                              const float (&v)[4], const uint32_t (&id)[4],
+                                              uint32_t* dbuf, int& dead_run, int lane) {
   const int cc = __popc(cm), dc = __popc(dm);
   int ci = cc, di = dc;
 #pragma unroll
@@ -544,12 +643,21 @@ __device__ __forceinline__ void record_events(const DevState& st, int g, int ins
     if (lane == 0) cbase = atomicAdd(st.cand_count, (unsigned)ctot);
     cbase = __shfl_sync(0xffffffffu, cbase, 0);
     unsigned w = cbase + (unsigned)(ci - cc);
+#pragma unroll
     for (int k2 = 0; k2 < 4; ++k2) {
       if (cm & (1u << k2)) {
-        if (w < (unsigned)st.cand_cap)
-          st.cand_buf[w] = ((unsigned long long)g << 32) | (unsigned long long)(off + 4 * q + k2);
-        else
+        if (w < (unsigned)st.cand_cap) {
+          if (kMany) {
+            st.cand_rec[w] = make_uint4((unsigned)(off + 4 * q + k2), id[k2],
+                                        __float_as_uint(z[k2]), __float_as_uint(v[k2]));
+            st.cand_seg[w] = (unsigned)g;
+          } else {
+            reinterpret_cast<unsigned long long*>(st.cand_rec)[w] =
+                ((unsigned long long)g << 32) | (unsigned long long)(off + 4 * q + k2);
+          }
+        } else {
           atomicOr(&st.dyn[inst].err, ERR_CAPACITY);
+        }
         ++w;
       }
     }
@@ -562,7 +670,7 @@ __device__ __forceinline__ void record_events(const DevState& st, int g, int ins
   }
 }
 
-template <bool kDepositOnly, int CQ>
+template <bool kDepositOnly, int CQ, bool kMany>
 __device__ __forceinline__ void push_body(const DevState& st) {
   constexpr int kChunkQuads = CQ, kArrBytes = CQ * 16, kStageBytes = stage_bytes(CQ);
   static_assert(CQ % 32 == 0 && CQ <= 128, "whole quads per lane");
@@ -830,8 +938,20 @@ __device__ __forceinline__ void push_body(const DevState& st) {
               deposit_quad(hist, z4, inv_dz, Nz);
             } else {
               const float zz[4] = {z4.x, z4.y, z4.z, z4.w};
-              deposit_warp(hist, zz, ~dm & 0xFu, inv_dz, Nz, agg);
-              if (evt) record_events(st, g, inst, off, q, cm, dm, dbuf, dead_run, lane);
+              if (kMany) {
+                // the events first: the velocities and ids are dead after them
+                const float vv[4] = {v4.x, v4.y, v4.z, v4.w};
+                const uint32_t ii[4] = {iA[h].x, iA[h].y, iA[h].z, iA[h].w};
+                if (evt)
+                  record_events<true>(st, g, inst, off, q, cm, dm, zz, vv, ii, dbuf, dead_run, lane);
+                deposit_warp(hist, zz, ~dm & 0xFu, inv_dz, Nz, agg);
+              } else {
+                const uint32_t none[4] = {0u, 0u, 0u, 0u};
+                deposit_warp(hist, zz, ~dm & 0xFu, inv_dz, Nz, agg);
+                if (evt)
+                  record_events<false>(st, g, inst, off, q, cm, dm, zz, zz, none, dbuf, dead_run,
+                                       lane);
+              }
             }
           }
         }
@@ -849,7 +969,8 @@ __device__ __forceinline__ void push_body(const DevState& st) {
         for (int h = 0; h < kChunkQuads / 32; ++h) {
           const int q = wq0 + kChunkQuads * ch + 32 * h + lane;
           unsigned dm = 0, cm = 0, am = 0;
-          float zz[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+          float zz[4] = {0.0f, 0.0f, 0.0f, 0.0f}, vv[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+          uint32_t ii[4] = {0u, 0u, 0u, 0u};
           if (q < wq1) {
             const int i = 4 * q;
             float4 z4s = make_float4(0.f, 0.f, 0.f, 0.f), v4s = z4s;
@@ -867,12 +988,14 @@ __device__ __forceinline__ void push_body(const DevState& st) {
               if (i + k2 < N) {
                 float zv = kDepositOnly ? zp[i + k2] : zq[k2];
                 if (!kDepositOnly) {
-                  float vv = vq[k2];
-                  const unsigned r = push_one(c, Es2, zv, vv, iq[k2]);
+                  float vn = vq[k2];
+                  const unsigned r = push_one(c, Es2, zv, vn, iq[k2]);
                   if (r & 1u) dm |= 1u << k2;
                   if (r & 2u) cm |= 1u << k2;
                   zp[i + k2] = zv;
-                  vzp[i + k2] = vv;
+                  vzp[i + k2] = vn;
+                  vv[k2] = vn;
+                  ii[k2] = iq[k2];
                 }
                 if (!(dm & (1u << k2))) {
                   zz[k2] = zv;
@@ -883,7 +1006,7 @@ __device__ __forceinline__ void push_body(const DevState& st) {
           }
           deposit_warp(hist, zz, am, inv_dz, Nz, agg);
           if (!kDepositOnly && __any_sync(0xffffffffu, (cm | dm) != 0u))
-            record_events(st, g, inst, off, q, cm, dm, dbuf, dead_run, lane);
+            record_events<kMany>(st, g, inst, off, q, cm, dm, zz, vv, ii, dbuf, dead_run, lane);
         }
         if (!kDepositOnly) {
           __syncwarp();
@@ -912,10 +1035,23 @@ __device__ __forceinline__ void push_body(const DevState& st) {
     st.bt[blockIdx.x] = (int)min(global_ns() - t_start, 2000000000ull);
 }
 
-// the push with 64-quad and with 32-quad warp chunks
-__global__ void __launch_bounds__(384, 2) k_push(DevState st) { push_body<false, 64>(st); }
-__global__ void __launch_bounds__(384, 2) k_push32(DevState st) { push_body<false, 32>(st); }
-__global__ void k_deposit(DevState st) { push_body<true, 64>(st); }
+// The push with 64-quad and with 32-quad warp chunks and in one block per SM,
+// each also for handles with many collision candidates (DevState::cand_many).
+__global__ void __launch_bounds__(384, 2) k_push(DevState st) { push_body<false, 64, false>(st); }
+__global__ void __launch_bounds__(384, 2) k_push32(DevState st) { push_body<false, 32, false>(st); }
+__global__ void __launch_bounds__(768, 1) k_push_wide(DevState st) {
+  push_body<false, 64, false>(st);
+}
+__global__ void __launch_bounds__(384, 2) k_push_many(DevState st) {
+  push_body<false, 64, true>(st);
+}
+__global__ void __launch_bounds__(384, 2) k_push32_many(DevState st) {
+  push_body<false, 32, true>(st);
+}
+__global__ void __launch_bounds__(768, 1) k_push_wide_many(DevState st) {
+  push_body<false, 64, true>(st);
+}
+__global__ void k_deposit(DevState st) { push_body<true, 64, false>(st); }
 
 // ------------------------------------------------------------------ field solve
 // Poisson with Dirichlet phi_0 = 0, phi_Nz = V (Sec. 2.1), solved exactly by
@@ -1359,7 +1495,10 @@ __device__ void mid_absorbed(const DevState& st, int g, int part, unsigned char*
 // Blocks [0, n_inst): field of diode b.  [n_inst, 4 n_inst): absorbed list
 // and tallies of segment b - n_inst.  Block 4 n_inst: re-weights the push
 // blocks for the next step.  The rest: the candidates' collisions.
-__global__ void __launch_bounds__(kPostThreads, 2) k_mid(DevState st) {
+// kMany: DevState::cand_many (its collisions in a kernel of their own, since
+// they need more registers than the other roles).
+template <bool kMany>
+__device__ __forceinline__ void mid_body(const DevState& st) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long wsl[64];
   __shared__ double wsd[64];
@@ -1376,9 +1515,13 @@ __global__ void __launch_bounds__(kPostThreads, 2) k_mid(DevState st) {
     // candidate k goes to block k mod nb, so the collisions' arithmetic is
     // spread over every collision block's SM
     const unsigned m = (unsigned)(b - 4 * nf - 1), nb = (unsigned)(gridDim.x - 4 * nf - 1);
-    mcc_candidates(st, threadIdx.x * nb + m, nb * blockDim.x);
+    if (kMany) mcc_many(st, threadIdx.x * nb + m, nb * blockDim.x, smem);
+    else mcc_few(st, threadIdx.x * nb + m, nb * blockDim.x);
   }
 }
+
+__global__ void __launch_bounds__(kPostThreads, 2) k_mid(DevState st) { mid_body<false>(st); }
+__global__ void __launch_bounds__(kPostThreads, 2) k_mid_many(DevState st) { mid_body<true>(st); }
 
 // Three blocks per diode, one per species: deterministic hole filling of the
 // species' absorbed slots (the ordered list k_mid left in dead_buf), then
