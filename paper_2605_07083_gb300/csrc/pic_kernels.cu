@@ -1523,6 +1523,16 @@ __device__ __forceinline__ void mid_body(const DevState& st) {
 __global__ void __launch_bounds__(kPostThreads, 2) k_mid(DevState st) { mid_body<false>(st); }
 __global__ void __launch_bounds__(kPostThreads, 2) k_mid_many(DevState st) { mid_body<true>(st); }
 
+// First of the n sorted slots that is >= x.
+__device__ __forceinline__ int lower_bound(const uint32_t* dd, int n, int x) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if ((int)dd[mid] < x) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
 // Three blocks per diode, one per species: deterministic hole filling of the
 // species' absorbed slots (the ordered list k_mid left in dead_buf), then
 // its appends -- thermionic electrons (species 0), ionisation children
@@ -1531,7 +1541,7 @@ __global__ void __launch_bounds__(kPostThreads, 2) k_mid_many(DevState st) { mid
 // count, ions absorbed).  The ion block also closes the diode's step (window
 // tallies, next id, step counter) as soon as it has the counts; no block
 // waits for another.
-__global__ void __launch_bounds__(kPostThreads, 1) k_post(DevState st) {
+__global__ void __launch_bounds__(kPostThreads, 2) k_post(DevState st) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int ws32[32];
   __shared__ InstConst ic;
@@ -1576,39 +1586,44 @@ __global__ void __launch_bounds__(kPostThreads, 1) k_post(DevState st) {
   }
   __syncthreads();                 // ic, the counts and the list are read by every thread below
   if (tid == 0) sNemit = emitted_count(ic, step);
-  if (sp == 2 && tid == 0) {
-    // ---- the diode's step closes here, while the blocks work on: window
-    // tallies, ids, step.  Nothing in this kernel reads what this writes
-    // (the step and first id come from PostScratch, the event count is
-    // reset by the next push).
-    const int Nem = sNemit, Ev = sE;
-    const int Pt = ic.replenish ? ps->D[2] : 0;
-    const uint32_t id_end = base_id + 2u * (uint32_t)Ev + (uint32_t)Nem + 2u * (uint32_t)Pt;
-    dyn->next_id = id_end;
-    // ids key the random streams: a diode that has handed out all 2^32 of
-    // them would reuse one, so that is reported as running out of capacity
-    if ((unsigned long long)base_id + 2ull * (unsigned)Ev + (unsigned)Nem + 2ull * (unsigned)Pt >
-        0xFFFFFFFFull)
-      atomicOr(&dyn->err, ERR_CAPACITY);
-    if (step >= ic.window_start) {
-      dyn->win_steps += 1;
-      for (int k = 0; k < 3; ++k)
-        for (int w = 0; w < 2; ++w) {
-          long long c = 0;
-          double e = 0.0;
-          for (int r = 0; r < st.kp; ++r) {       // k_mid's list blocks, in order
-            c += ps->cnt[k][r][w];
-            e += ps->ke[k][r][w];
-          }
-          dyn->count[k][w] += c;
-          dyn->ke[k][w] += e;
-        }
-      dyn->emitted += Nem;
-      dyn->replenished += Pt;
+  if (sp == 2 && tid >= nt - 32) {
+    // ---- the diode's step closes here, in a warp that has no hole to fill
+    // on a normal step: window tallies (a lane per species and electrode; the
+    // FP64 adds of kp parts take ~0.1 us each), ids, step.  Nothing in this
+    // kernel reads what this writes (the step and first id come from
+    // PostScratch, the event count is reset by the next push).
+    const int lane = tid & 31;
+    const bool in_win = step >= ic.window_start;
+    if (lane < 6 && in_win) {
+      const int k = lane >> 1, w = lane & 1;
+      long long c = 0;
+      double e = 0.0;
+      for (int r = 0; r < st.kp; ++r) {       // k_mid's list blocks, in order
+        c += ps->cnt[k][r][w];
+        e += ps->ke[k][r][w];
+      }
+      dyn->count[k][w] += c;
+      dyn->ke[k][w] += e;
     }
-    dyn->pushed += (long long)ps->N[0] + ps->N[1] + ps->N[2];
-    dyn->emit_dep = 0;
-    dyn->step = step + 1;
+    if (lane == 31) {
+      const int Nem = emitted_count(ic, step), Ev = sE;
+      const int Pt = ic.replenish ? ps->D[2] : 0;
+      const uint32_t id_end = base_id + 2u * (uint32_t)Ev + (uint32_t)Nem + 2u * (uint32_t)Pt;
+      dyn->next_id = id_end;
+      // ids key the random streams: a diode that has handed out all 2^32 of
+      // them would reuse one, so that is reported as running out of capacity
+      if ((unsigned long long)base_id + 2ull * (unsigned)Ev + (unsigned)Nem + 2ull * (unsigned)Pt >
+          0xFFFFFFFFull)
+        atomicOr(&dyn->err, ERR_CAPACITY);
+      if (in_win) {
+        dyn->win_steps += 1;
+        dyn->emitted += Nem;
+        dyn->replenished += Pt;
+      }
+      dyn->pushed += (long long)ps->N[0] + ps->N[1] + ps->N[2];
+      dyn->emit_dep = 0;
+      dyn->step = step + 1;
+    }
   }
   if (sp == 2) {
     // every k_mid field block has read the push's charge: clear it for the
@@ -1618,75 +1633,48 @@ __global__ void __launch_bounds__(kPostThreads, 1) k_post(DevState st) {
   }
 
   // ---- hole filling: the dead slots below the new count take the live
-  // particles above it, in order.  The species-0 block draws its first
-  // emitted electrons while the first round's loads are in flight.
+  // particles above it, in order.  The listed slots are sorted, so a tail
+  // slot's rank among the live ones follows from its place among the listed:
+  // no scan, and sources (>= Nn) and holes (< Nn) are disjoint.  (With a block
+  // scan over the tail, the close below in the same thread and one block per SM
+  // the kernel took 0.5 us longer on one diode, 5 us on 128.)  The
+  // species-0 block draws its first emitted electrons while the first loads
+  // are in flight.
   const int Nn = N - D;
   constexpr int kEmitRegs = 2;
   float ez[kEmitRegs], evx[kEmitRegs], evy[kEmitRegs], evz[kEmitRegs];
   bool have_emit = false;
-  {
-    int lo = 0, hi = D;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if ((int)dd[mid] < Nn) lo = mid + 1; else hi = mid;
-    }
-    const int h = lo;
-    // kPer consecutive tail slots per thread: one search, one block scan and
-    // one gather-then-scatter round trip for up to kPer * nt of them
-    constexpr int kPer = 4;
-    int run = 0;
-    for (int base = 0; base < D; base += kPer * nt) {
-      const int k0 = base + kPer * tid;
-      const int t0 = Nn + k0;
-      int a2 = h, b2 = D;                        // first listed slot >= t0
-      while (a2 < b2) {
-        const int mid = (a2 + b2) >> 1;
-        if ((int)dd[mid] < t0) a2 = mid + 1; else b2 = mid;
-      }
-      unsigned lm = 0u;
-      int cnt = 0;
-#pragma unroll
-      for (int u = 0; u < kPer; ++u) {
-        if (k0 + u < D) {
-          if (a2 < D && (int)dd[a2] == t0 + u) {
-            ++a2;                                // absorbed: not moved
-          } else {
-            lm |= 1u << u;
-            ++cnt;
-          }
+  if (D > 0) {
+    const int h = lower_bound(dd, D, Nn);        // holes: the listed slots below Nn
+    for (int k = tid; k < D || k == tid; k += nt) {
+      const int t0 = Nn + k;
+      int to = -1;
+      float z, vx, vy, vz;
+      uint32_t id;
+      if (k < D) {
+        const int a2 = lower_bound(dd, D, t0);   // listed slots before the tail slot
+        if (a2 == D || (int)dd[a2] != t0) {
+          to = (int)dd[k - (a2 - h)];            // the hole of the same rank
+          const long long src = off + t0;
+          z = st.z[src];
+          vx = st.vx[src];
+          vy = st.vy[src];
+          vz = st.vz[src];
+          id = st.id[src];
         }
       }
-      int tot;
-      int r = block_exclusive_scan<int>(cnt, &tot, ws32) + run;
-      float z[kPer], vx[kPer], vy[kPer], vz[kPer];
-      uint32_t id[kPer];
-#pragma unroll
-      for (int u = 0; u < kPer; ++u) {
-        if (lm & (1u << u)) {
-          const long long src = off + t0 + u;
-          z[u] = st.z[src];
-          vx[u] = st.vx[src];
-          vy[u] = st.vy[src];
-          vz[u] = st.vz[src];
-          id[u] = st.id[src];
-        }
-      }
-      if (sp == 0 && base == 0) {
-        const int Ne = sNemit;                   // written before the scan's barriers
+      if (sp == 0 && k == tid) {
+        const int Ne = emitted_count(ic, step);
 #pragma unroll
         for (int j = 0; j < kEmitRegs; ++j)
           if (tid + j * nt < Ne)
             emitted_electron(ic, tid + j * nt, step, ez[j], evx[j], evy[j], evz[j]);
         have_emit = true;
       }
-#pragma unroll
-      for (int u = 0; u < kPer; ++u) {
-        if (lm & (1u << u)) put_particle(st, off, dd[r++], z[u], vx[u], vy[u], vz[u], id[u]);
-      }
-      run += tot;
+      if (to >= 0) put_particle(st, off, to, z, vx, vy, vz, id);
     }
-    __syncthreads();                 // shared memory is reused below
   }
+  __syncthreads();                   // tail slots are read, shared memory is reused below
 
   // ---- appends of this species (their charge is in the field already)
   const int E = sE, Nemit = sNemit;
