@@ -26,6 +26,10 @@ __global__ void k_deposit(DevState st);
 __global__ void k_mid(DevState st);
 __global__ void k_mid_many(DevState st);
 __global__ void k_post(DevState st);
+__global__ void k_fused(DevState st, int n_steps);
+__global__ void k_route(DevState st, int C, int sms, long long growth,
+                        cudaGraphConditionalHandle handle);
+size_t fused_smem_bytes(int nodes);
 __global__ void k_field(DevState st);
 __global__ void k_profile(DevState st);
 __global__ void k_phi(DevState st);
@@ -91,6 +95,8 @@ struct pic_handle {
   int* inject_flag = nullptr;   // device word: an injected z outside [0, L)
   int bw_len = 0;
   int mcc_blocks = 0;
+  int fused_c = 0;              // blocks per diode of k_fused (0: not taken)
+  size_t fused_smem = 0;
   bool sort_ready = false;
   SortGrid sort_grid{1, 1, 1};
   int prof_gx = 1;              // k_profile blocks per segment
@@ -275,7 +281,7 @@ cudaError_t raise_smem_limits(int device) {
                        (const void*)k_push_wide_many,
                        (const void*)k_deposit, (const void*)k_field,
                        (const void*)k_post, (const void*)k_profile, (const void*)k_phi,
-                       (const void*)k_mid, (const void*)k_mid_many};
+                       (const void*)k_mid, (const void*)k_mid_many, (const void*)k_fused};
   for (const void* f : fns) {
     e = set_dynamic_smem_limit(f, optin);
 
@@ -344,6 +350,8 @@ void default_push_shape(pic_handle* h) {
   h->push_threads = best_t;
   h->push_chunk = best_c;
 }
+
+void set_fused_shape(pic_handle* h);
 
 int set_launch_shape(pic_handle* h) {
   cudaError_t e = raise_smem_limits(h->device);
@@ -448,6 +456,7 @@ int set_launch_shape(pic_handle* h) {
                                           std::max<int64_t>(1, 2 * h->sm_count / h->n_seg));
   h->prof_gx = (int)std::max<int64_t>(1, std::max(gmin, gfill));
   h->prof_smem = (size_t)(h->max_nodes - 1) * 12;
+  set_fused_shape(h);
   drop_graph(h);
   return PIC_OK;
 }
@@ -527,24 +536,135 @@ cudaError_t launch_step(pic_handle* h) {
   return cudaGetLastError();
 }
 
+// the three kernels of n steps (and what follows them) on the handle's stream
+void enqueue_steps(pic_handle* h, int n, int first) {
+  for (int i = 0; i < n; ++i) {
+    push_kernel(h, h->push_threads, h->push_chunk)<<<h->G, h->push_threads, h->push_smem,
+                                                    h->stream>>>(h->st);
+    mid_kernel(h)<<<mid_blocks(h), kPostThreads, h->mid_smem, h->stream>>>(h->st);
+    k_post<<<3 * h->n_inst, kPostThreads, h->post_smem, h->stream>>>(h->st);
+    launch_profile(h);
+    if (sort_due(h, first + i + 1)) launch_sort(h);
+  }
+}
+
+cudaError_t enqueue_fused(pic_handle* h, int n) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(h->n_inst * h->fused_c));
+  cfg.blockDim = dim3(kFusedThreads);
+  cfg.dynamicSmemBytes = h->fused_smem;
+  cfg.stream = h->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)h->fused_c;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_fused, h->st, n);
+}
+
+// Blocks per diode of k_fused: as many as let all clusters be resident at
+// once, a power of two up to the portable cluster size; 0 where a block does
+// not fit (its shared memory grows with the cells).
+void set_fused_shape(pic_handle* h) {
+  h->fused_c = 0;
+  h->fused_smem = fused_smem_bytes(h->max_nodes);
+  for (int c = 8; c >= 1 && h->fused_c == 0; c /= 2) {
+    if (c > 1 && h->n_inst * c > h->sm_count) continue;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(h->n_inst * c));
+    cfg.blockDim = dim3(kFusedThreads);
+    cfg.dynamicSmemBytes = h->fused_smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)c;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_fused, &cfg) == cudaSuccess &&
+        n >= (c > 1 ? h->n_inst : 1))
+      h->fused_c = c;
+  }
+  cudaGetLastError();                  // a shape that does not fit is no error
+}
+
+// k_fused takes neither sorts nor profile samples, and has no bulk-copy wait
+// to give up on
+bool fused_allowed(const pic_handle* h) {
+  return h->fused_c > 0 && h->sort_period <= 0 && h->st.prof_period <= 0 &&
+         h->st.wait_limit == kWaitLimit;
+}
+
+// Steps per decision between k_fused and the three kernels
+constexpr int kRouteSteps = 64;
+
+// n steps by the way k_route picks on the device, as nodes of g after *tail
+int add_routed_steps(pic_handle* h, cudaGraph_t g, int n, cudaGraphNode_t* tail) {
+  cudaGraphConditionalHandle cond;
+  cudaError_t e = cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault);
+  if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaGraphConditionalHandleCreate");
+  // most a diode can gain: its emission, and two particles per ionisation event
+  long long growth = 0;
+  for (const InstConst& k : h->ic)
+    growth = std::max(growth, (long long)n * (k.emit_floor + 1 + 2 * kEvCap));
+  int C = h->fused_c, sms = h->sm_count;
+  void* args[] = {&h->st, &C, &sms, &growth, &cond};
+  cudaKernelNodeParams kp = {};
+  kp.func = (void*)k_route;
+  kp.gridDim = dim3(1);
+  kp.blockDim = dim3(256);
+  kp.kernelParams = args;
+  cudaGraphNode_t route;
+  e = cudaGraphAddKernelNode(&route, g, *tail ? tail : nullptr, *tail ? 1 : 0, &kp);
+  if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaGraphAddKernelNode");
+  cudaGraphNodeParams cp = {};
+  cp.type = cudaGraphNodeTypeConditional;
+  cp.conditional.handle = cond;
+  cp.conditional.type = cudaGraphCondTypeIf;
+  cp.conditional.size = 2;             // then and else
+  e = cudaGraphAddNode(tail, g, &route, nullptr, 1, &cp);
+  if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaGraphAddNode");
+  for (int body = 0; body < 2; ++body) {
+    e = cudaStreamBeginCaptureToGraph(h->stream, cp.conditional.phGraph_out[body], nullptr, nullptr,
+                                      0, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaStreamBeginCaptureToGraph");
+    cudaError_t launched = cudaSuccess;
+    if (body == 0) launched = enqueue_fused(h, n);
+    else enqueue_steps(h, n, 0);
+    cudaGraph_t captured = nullptr;
+    e = cudaStreamEndCapture(h->stream, &captured);
+    if (e == cudaSuccess) e = launched;
+    if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaStreamEndCapture");
+  }
+  return PIC_OK;
+}
+
 // Captures len steps.  With a periodic sort the graph is only ever launched
 // on a sort-aligned step, so the sorts sit after every sort_period-th step of
 // it counted from its start.
 int build_graph(pic_handle* h, int len, cudaGraphExec_t* out) {
   *out = nullptr;
   cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
-  if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaStreamBeginCapture");
-  for (int i = 0; i < len; ++i) {
-    push_kernel(h, h->push_threads, h->push_chunk)<<<h->G, h->push_threads, h->push_smem, h->stream>>>(h->st);
-    mid_kernel(h)<<<mid_blocks(h), kPostThreads, h->mid_smem, h->stream>>>(h->st);
-    k_post<<<3 * h->n_inst, kPostThreads, h->post_smem, h->stream>>>(h->st);
-    launch_profile(h);
-    if (sort_due(h, i + 1)) launch_sort(h);
+  if (fused_allowed(h) && len >= kFusedMinSteps) {
+    cudaError_t e = cudaGraphCreate(&g, 0);
+    if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaGraphCreate");
+    cudaGraphNode_t tail = nullptr;
+    for (int s = 0; s < len; s += kRouteSteps) {
+      int rc = add_routed_steps(h, g, std::min(kRouteSteps, len - s), &tail);
+      if (rc != PIC_OK) {
+        cudaGraphDestroy(g);
+        return rc;
+      }
+    }
+  } else {
+    cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaStreamBeginCapture");
+    enqueue_steps(h, len, 0);
+    e = cudaStreamEndCapture(h->stream, &g);
+    if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaStreamEndCapture");
   }
-  e = cudaStreamEndCapture(h->stream, &g);
-  if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaStreamEndCapture");
-  e = cudaGraphInstantiate(out, g, 0);
+  cudaError_t e = cudaGraphInstantiate(out, g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) {
     *out = nullptr;

@@ -30,7 +30,15 @@ constexpr uint32_t kStreamInject = 3;
 // sticky error bits: bit (-code - 1)
 enum ErrBit : int32_t { ERR_CAPACITY = 1 << 3, ERR_TIMEOUT = 1 << 4, ERR_ENERGYCAP = 1 << 5 };
 
-constexpr int kMccThreads = 256;
+constexpr int kFusedThreads = 512;      // threads per block of k_fused
+constexpr int kFusedMinSteps = 8;      // shortest graph that lets k_route choose
+// k_route's estimate of a step's time, ns: the fused kernel's fixed part, per
+// block of the cluster and per cell, and its particles per ns and block; the
+// three kernels' fixed part, per diode, and particles per ns (fits to the
+// measured steps of 1 to 512 diodes of 128 to 2000 cells)
+constexpr float kFusedStepNs = 7700.0f, kFusedBlockNs = 40.0f, kFusedCellNs = 3.5f;
+constexpr float kFusedRate = 1.8f;
+constexpr float kThreeStepNs = 16000.0f, kThreeDiodeNs = 95.0f, kThreeRate = 270.0f;
 
 // Per-instance constants, derived on the host in FP64 and stored once.
 struct InstConst {

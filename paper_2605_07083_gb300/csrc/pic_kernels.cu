@@ -452,6 +452,25 @@ __device__ __forceinline__ void emitted_electron(const InstConst& ic, int k, lon
   vy = ic.sig_w * n1;
 }
 
+// Replenished pair k of a step (Sec. 2.1): a common uniform position, the
+// electron's or the ion's Maxwellian velocity.
+__device__ __forceinline__ void replenished(const InstConst& ic, int k, long long step, bool ion,
+                                            float& z, float& vx, float& vy, float& vz) {
+  const uint4 A = philox10(make_uint4((uint32_t)k, (uint32_t)step, 0u, TAG_REPL),
+                           ic.key0[kStreamInject], ic.key1);
+  const uint4 B = philox10(make_uint4((uint32_t)k, (uint32_t)step, 1u, TAG_REPL),
+                           ic.key0[kStreamInject], ic.key1);
+  float gg[6];
+  box_muller(A.x, A.y, gg[0], gg[1]);
+  box_muller(A.z, A.w, gg[2], gg[3]);
+  box_muller(B.x, B.y, gg[4], gg[5]);
+  const float sig = ion ? ic.sig_i0 : ic.sig_e0;
+  z = u01f(B.z) * ic.L_f;
+  vx = sig * (ion ? gg[3] : gg[0]);
+  vy = sig * (ion ? gg[4] : gg[1]);
+  vz = sig * (ion ? gg[5] : gg[2]);
+}
+
 // ------------------------------------------------------------------ k_push
 struct SegCtx {
   float inv_dz, Lf, dt, qmdt;
@@ -1723,23 +1742,12 @@ __global__ void __launch_bounds__(kPostThreads, 2) k_post(DevState st) {
     }
     // replenishment (Sec. 2.1): one e-ion pair at a common uniform position
     // per ion absorbed; both blocks draw the pair's numbers
-    const float sig = (sp == 2) ? ic.sig_i0 : ic.sig_e0;
     for (int k = tid; k < P; k += nt) {
-      const uint4 A = philox10(make_uint4((uint32_t)k, (uint32_t)step, 0u, TAG_REPL), ic.key0[kStreamInject], ic.key1);
-      const uint4 B = philox10(make_uint4((uint32_t)k, (uint32_t)step, 1u, TAG_REPL), ic.key0[kStreamInject], ic.key1);
-      float gg[6];
-      box_muller(A.x, A.y, gg[0], gg[1]);
-      box_muller(A.z, A.w, gg[2], gg[3]);
-      box_muller(B.x, B.y, gg[4], gg[5]);
-      const float z = u01f(B.z) * ic.L_f;
+      float z, vx, vy, vz;
+      replenished(ic, k, step, sp == 2, z, vx, vy, vz);
       const long long sl = (long long)Nn + E + k;
-      if (sl < cap) {
-        const bool ion = sp == 2;
-        put_particle(st, off, sl, z, sig * (ion ? gg[3] : gg[0]), sig * (ion ? gg[4] : gg[1]),
-                     sig * (ion ? gg[5] : gg[2]), id_repl + 2u * k + idb);
-      } else {
-        overflow = true;
-      }
+      if (sl < cap) put_particle(st, off, sl, z, vx, vy, vz, id_repl + 2u * k + idb);
+      else overflow = true;
     }
     newN = min(Nn + E + P, cap);
   }
@@ -1799,3 +1807,5 @@ __global__ void k_count_outside(const float* z, long long n, float Lf, int* bad)
 }
 
 }  // namespace pic
+
+#include "pic_fused.cuh"
