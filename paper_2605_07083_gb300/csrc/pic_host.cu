@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "../../include/pic.h"
@@ -32,9 +33,16 @@ __global__ void k_route(DevState st, int C, int sms, long long growth,
 size_t fused_smem_bytes(int nodes);
 __global__ void k_field(DevState st);
 __global__ void k_profile(DevState st);
-__global__ void k_phi(DevState st);
-__global__ void k_fill_ids(uint32_t* id, long long n, uint32_t first);
-__global__ void k_count_outside(const float* z, long long n, float Lf, int* bad);
+__global__ void k_phi(DevState st, int inst, Readback* out);
+__global__ void k_read(DevState st, int inst, Readback* out);
+__global__ void k_read_rho(DevState st, int inst, Readback* out);
+__global__ void k_state_copy(DevState st, int g, long long cap, float* z, float* vx, float* vy,
+                             float* vz, uint32_t* id, int vec, Readback* out);
+__global__ void k_inject(DevState st, long long at, long long n, const float* zs, const float* vxs,
+                         const float* vys, const float* vzs, uint32_t first, float Lf, int vec,
+                         int* bad);
+__global__ void k_inject_commit(DevState st, int g, int count, uint32_t next_id, int* bad,
+                                Readback* out);
 void sort_launch(const DevState& st, const SortGrid& r, int max_nz, cudaStream_t s);
 int sort_slots(int sms, int n_seg, int max_nz);
 size_t sort_hist_ints(const int32_t* seg_cap, const int* seg_nz, int n_seg, int slots,
@@ -93,6 +101,11 @@ struct pic_handle {
   size_t dcount_ints = 0;
   int bstart_len = 0;
   int* inject_flag = nullptr;   // device word: an injected z outside [0, L)
+  Readback* rb = nullptr;       // mapped host memory the reading kernels write
+  // live counts and next ids while no step has run since they were known
+  bool counts_known = false;
+  std::vector<int32_t> known_count;
+  std::vector<uint32_t> known_id;
   int bw_len = 0;
   int mcc_blocks = 0;
   int fused_c = 0;              // blocks per diode of k_fused (0: not taken)
@@ -235,20 +248,81 @@ int64_t default_capacity(const pic_config& c, int s) {
   return 1 << 20;
 }
 
-int check_flags(pic_handle* h) {
-  std::vector<InstDyn> dyn(h->n_inst);
-  cudaError_t e = cudaMemcpyAsync(dyn.data(), h->st.dyn, sizeof(InstDyn) * h->n_inst,
-                                  cudaMemcpyDeviceToHost, h->stream);
+// Mapped host memory for the readbacks.  Pinning a block costs more than a
+// small run's reads, so a destroyed handle's block is kept for the next one,
+// at most kReadPool of them (5 MB); each block belongs to one handle at a time.
+constexpr size_t kReadPool = 64;
+std::mutex g_read_mu;
+std::vector<Readback*> g_read_free;
+
+Readback* readback_take() {
+  {
+    std::lock_guard<std::mutex> lock(g_read_mu);
+    if (!g_read_free.empty()) {
+      Readback* r = g_read_free.back();
+      g_read_free.pop_back();
+      return r;
+    }
+  }
+  void* p = nullptr;
+  if (cudaHostAlloc(&p, kReadBytes, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess)
+    return nullptr;
+  return (Readback*)p;
+}
+
+void readback_give(Readback* r) {
+  if (!r) return;
+  {
+    std::lock_guard<std::mutex> lock(g_read_mu);
+    if (g_read_free.size() < kReadPool) {
+      g_read_free.push_back(r);
+      return;
+    }
+  }
+  cudaFreeHost(r);
+}
+
+// wait for the readback kernel just launched
+int read_done(pic_handle* h) {
+  cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  int bits = 0;
-  for (auto& d : dyn) bits |= d.err;
+  return e == cudaSuccess ? PIC_OK : cuda_fail(h, e);
+}
+
+// the sticky code after a readback
+int flags_of(pic_handle* h) {
+  const int bits = h->rb->err;
   if (h->sticky == PIC_OK) {
     if (bits & ERR_CAPACITY) h->sticky = PIC_ECAPACITY;
     else if (bits & ERR_TIMEOUT) h->sticky = PIC_ETIMEOUT;
     else if (bits & ERR_ENERGYCAP) h->sticky = PIC_EENERGYCAP;
   }
   return h->sticky;
+}
+
+int check_flags(pic_handle* h) {
+  k_read<<<1, 256, 0, h->stream>>>(h->st, -1, h->rb);
+  int rc = read_done(h);
+  return rc == PIC_OK ? flags_of(h) : rc;
+}
+
+// Device arrays that a kernel may read or write: device or managed memory,
+// aligned to their elements.  Anything else goes through cudaMemcpyAsync,
+// which handles it or refuses it.  *vec: all are 16-byte aligned.
+bool kernel_arrays(std::initializer_list<const void*> ps, bool* vec) {
+  *vec = true;
+  for (const void* p : ps) {
+    if (!p) continue;
+    if ((uintptr_t)p & 3u) return false;
+    if ((uintptr_t)p & 15u) *vec = false;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (a.type != cudaMemoryTypeDevice && a.type != cudaMemoryTypeManaged) return false;
+  }
+  return true;
 }
 
 void drop_graph(pic_handle* h) {
@@ -532,6 +606,7 @@ cudaError_t launch_step(pic_handle* h) {
   k_post<<<3 * h->n_inst, kPostThreads, h->post_smem, h->stream>>>(h->st);
   launch_profile(h);
   h->host_step += 1;
+  h->counts_known = false;
   if (sort_due(h, h->host_step)) launch_sort(h);
   return cudaGetLastError();
 }
@@ -848,23 +923,37 @@ int pic_create(const pic_config* cfgs, int n_instances, void* cuda_stream,
   st.n_seg = h->n_seg;
   st.max_nodes = h->max_nodes;
   const size_t P = (size_t)h->total_cap;
-  void* p[16] = {nullptr};
-  p[0] = dev_alloc(h, P * 4); p[1] = dev_alloc(h, P * 4); p[2] = dev_alloc(h, P * 4);
-  p[3] = dev_alloc(h, P * 4); p[4] = dev_alloc(h, P * 4);
-  p[5] = dev_alloc(h, P * 4); p[6] = dev_alloc(h, P * 4);
-  p[7] = dev_alloc(h, sizeof(int64_t) * h->n_seg);
-  p[8] = dev_alloc(h, sizeof(int32_t) * h->n_seg * 2);
-  p[9] = dev_alloc(h, sizeof(int64_t) * (h->n_seg + 2));
-  p[10] = dev_alloc(h, sizeof(Event) * (size_t)kEvCap * h->n_inst);
-  p[11] = dev_alloc(h, sizeof(int64_t) * nodes * 2 + sizeof(double) * nodes + sizeof(float) * nodes);
-  p[12] = dev_alloc(h, sizeof(InstConst) * h->n_inst);
-  p[13] = dev_alloc(h, sizeof(InstDyn) * h->n_inst);
   // candidates per step: far above the expected P_cand * N (<= 1e-2 of all slots)
   const int64_t cand_cap = std::min<int64_t>(h->total_cap / 16 + 65536, 1LL << 30);
-  p[14] = dev_alloc(h, (sizeof(uint4) + sizeof(uint32_t)) * (size_t)cand_cap + 256);
-  p[15] = dev_alloc(h, sizeof(PostScratch) * h->n_inst);
-  for (int k = 0; k < 16; ++k)
+  // sizes of the handle's arrays, one allocation for all (an allocator's
+  // callback costs several microseconds a call) or, if no block that large is
+  // to be had, one each
+  const size_t need[17] = {
+      P * 4, P * 4, P * 4, P * 4, P * 4, P * 4, P * 4,
+      sizeof(int64_t) * h->n_seg, sizeof(int32_t) * h->n_seg * 2, sizeof(int64_t) * (h->n_seg + 2),
+      sizeof(Event) * (size_t)kEvCap * h->n_inst,
+      sizeof(int64_t) * nodes * 2 + sizeof(double) * nodes + sizeof(float) * nodes,
+      sizeof(InstConst) * h->n_inst, sizeof(InstDyn) * h->n_inst,
+      (sizeof(uint4) + sizeof(uint32_t)) * (size_t)cand_cap + 256,
+      sizeof(PostScratch) * h->n_inst, sizeof(int)};
+  void* p[17] = {nullptr};
+  size_t all = 0;
+  for (size_t b : need) all += (b + 255) & ~(size_t)255;
+  if (char* block = (char*)dev_alloc(h, all)) {
+    size_t at = 0;
+    for (int k = 0; k < 17; ++k) {
+      p[k] = block + at;
+      at += (need[k] + 255) & ~(size_t)255;
+    }
+  } else {
+    cudaGetLastError();
+    for (int k = 0; k < 17; ++k) p[k] = dev_alloc(h, need[k]);
+  }
+  for (int k = 0; k < 17; ++k)
     if (!p[k]) { pic_destroy(h); return PIC_ENOMEM; }
+  h->inject_flag = (int*)p[16];
+  h->rb = readback_take();
+  if (!h->rb) { pic_destroy(h); return PIC_ENOMEM; }
   st.z = (float*)p[0]; st.vx = (float*)p[1]; st.vy = (float*)p[2]; st.vz = (float*)p[3];
   st.id = (uint32_t*)p[4];
   st.dead_buf = (uint32_t*)p[5];
@@ -904,6 +993,10 @@ int pic_create(const pic_config* cfgs, int n_instances, void* cuda_stream,
   if (e == cudaSuccess) e = cudaMemsetAsync(st.part, 0, sizeof(int64_t) * (h->n_seg + 2), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(st.cand_count, 0, sizeof(unsigned int), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(st.post, 0, sizeof(PostScratch) * h->n_inst, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->inject_flag, 0, sizeof(int), h->stream);
+  h->counts_known = true;
+  h->known_count.assign(h->n_seg, 0);
+  h->known_id.assign(h->n_inst, 0u);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) { pic_destroy(h); return PIC_ECUDA; }
   int rc = set_launch_shape(h);
@@ -920,49 +1013,43 @@ int pic_inject(pic_handle* h, int instance, int species, int64_t n, const float*
   if (!z || !vx || !vy || !vz) return PIC_EINVAL;
   const int g = 3 * instance + species;
   const float Lf = h->ic[instance].L_f;
-  int32_t count = 0;
-  InstDyn d;
-  cudaError_t e = cudaMemcpyAsync(&count, h->st.seg_count + g, sizeof(int32_t),
-                                  cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&d, h->st.dyn + instance, sizeof(InstDyn), cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  if ((int64_t)count + n > h->seg_cap[g]) return PIC_ECAPACITY;
-  if (!h->inject_flag) {
-    h->inject_flag = (int*)dev_alloc(h, sizeof(int));
-    if (!h->inject_flag) return PIC_ENOMEM;
+  if (!h->counts_known) {
+    k_read<<<1, 256, 0, h->stream>>>(h->st, instance, h->rb);
+    int rc = read_done(h);
+    if (rc != PIC_OK) return rc;
   }
+  const int32_t count = h->counts_known ? h->known_count[g] : h->rb->count[species];
+  const uint32_t next_id = h->counts_known ? h->known_id[instance] : h->rb->dyn.next_id;
+  if ((int64_t)count + n > h->seg_cap[g]) return PIC_ECAPACITY;
   // the particles go into the free slots after the live ones and their z
   // is checked there, on the device; they are counted in only if every z
   // lies in [0, L), so a rejected call leaves the instance as it was
   const int64_t base = h->seg_off[g] + count;
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  const size_t bytes = sizeof(float) * (size_t)n;
-  e = cudaMemcpyAsync(h->st.z + base, z, bytes, kind, h->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->st.vx + base, vx, bytes, kind, h->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->st.vy + base, vy, bytes, kind, h->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->st.vz + base, vz, bytes, kind, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->inject_flag, 0, sizeof(int), h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  const unsigned blocks = (unsigned)((n + 255) / 256);
-  k_count_outside<<<blocks, 256, 0, h->stream>>>(h->st.z + base, n, Lf, h->inject_flag);
-  k_fill_ids<<<blocks, 256, 0, h->stream>>>(h->st.id + base, n, d.next_id);
-  int hb = 0;
-  e = cudaGetLastError();
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&hb, h->inject_flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  if (hb) return PIC_EINVAL;
+  bool vec = true;
+  const bool direct = on_device && kernel_arrays({z, vx, vy, vz}, &vec);
+  if (!direct) {
+    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    const size_t bytes = sizeof(float) * (size_t)n;
+    cudaError_t e = cudaMemcpyAsync(h->st.z + base, z, bytes, kind, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->st.vx + base, vx, bytes, kind, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->st.vy + base, vy, bytes, kind, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->st.vz + base, vz, bytes, kind, h->stream);
+    if (e != cudaSuccess) return cuda_fail(h, e);
+    vec = true;
+  }
+  const unsigned blocks = (unsigned)((n + 1023) / 1024);
   const int32_t newc = (int32_t)(count + n);
-  const uint32_t nid = d.next_id + (uint32_t)n;
-  e = cudaMemcpyAsync(h->st.seg_count + g, &newc, sizeof(int32_t), cudaMemcpyHostToDevice, h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&h->st.dyn[instance].next_id, &nid, sizeof(uint32_t), cudaMemcpyHostToDevice,
-                        h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
+  const uint32_t nid = next_id + (uint32_t)n;
+  k_inject<<<blocks, 256, 0, h->stream>>>(h->st, base, n, direct ? z : nullptr, vx, vy, vz, next_id,
+                                          Lf, vec && base % 4 == 0 ? 1 : 0, h->inject_flag);
+  k_inject_commit<<<1, 1, 0, h->stream>>>(h->st, g, newc, nid, h->inject_flag, h->rb);
+  int rc = read_done(h);
+  if (rc != PIC_OK) return rc;
+  if (h->rb->bad) return PIC_EINVAL;
+  if (h->counts_known) {
+    h->known_count[g] = newc;
+    h->known_id[instance] = nid;
+  }
   h->dirty = true;
   return PIC_OK;
 }
@@ -1012,6 +1099,7 @@ static int step_plan(pic_handle* h, int64_t n_steps, bool run) {
       }
       while (left >= g.first) {
         if (run) {
+          h->counts_known = false;
           cudaError_t e = cudaGraphLaunch(g.second, h->stream);
           if (e != cudaSuccess) return cuda_fail(h, e);
           h->host_step += g.first;
@@ -1049,6 +1137,7 @@ int pic_profile_steps(pic_handle* h, int64_t n_steps, pic_profile* out) {
   std::memset(out, 0, sizeof(*out));
   int rc = ensure_field(h);
   if (rc != PIC_OK) return rc;
+  h->counts_known = false;
   std::vector<cudaEvent_t> ev(6 * (size_t)std::max<int64_t>(n_steps, 1));
   for (auto& x : ev) cudaEventCreate(&x);
   cudaEvent_t t0, t1;
@@ -1106,17 +1195,11 @@ int pic_profile_steps(pic_handle* h, int64_t n_steps, pic_profile* out) {
 
 int pic_diagnostics(pic_handle* h, int instance, pic_diag* out) {
   if (!h || !out || instance < 0 || instance >= h->n_inst) return PIC_EINVAL;
-  InstDyn d;
-  int32_t counts[3];
-  cudaError_t e = cudaMemcpyAsync(&d, h->st.dyn + instance, sizeof(InstDyn), cudaMemcpyDeviceToHost,
-                                  h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(counts, h->st.seg_count + 3 * instance, sizeof(counts),
-                        cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  fill_diag(h, instance, d, counts, out);
-  return check_flags(h);
+  k_read<<<1, 256, 0, h->stream>>>(h->st, instance, h->rb);
+  int rc = read_done(h);
+  if (rc != PIC_OK) return rc;
+  fill_diag(h, instance, h->rb->dyn, h->rb->count, out);
+  return flags_of(h);
 }
 
 int pic_get_state(pic_handle* h, int instance, int species, float* z, float* vx, float* vy,
@@ -1124,26 +1207,37 @@ int pic_get_state(pic_handle* h, int instance, int species, float* z, float* vx,
   if (!h || !n || instance < 0 || instance >= h->n_inst || species < 0 || species > 2)
     return PIC_EINVAL;
   const int g = 3 * instance + species;
-  int32_t count = 0;
-  cudaError_t e = cudaMemcpyAsync(&count, h->st.seg_count + g, sizeof(int32_t),
-                                  cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
+  bool vec = false;
+  if (on_device && kernel_arrays({z, vx, vy, vz, id}, &vec)) {
+    const int64_t room = std::max<int64_t>(1, std::min<int64_t>(cap, h->seg_cap[g]));
+    const unsigned blocks =
+        (unsigned)std::min<int64_t>((room + 1023) / 1024, (int64_t)8 * h->sm_count);
+    k_state_copy<<<blocks, 256, 0, h->stream>>>(h->st, g, cap, z, vx, vy, vz, id, vec ? 1 : 0, h->rb);
+    int rc = read_done(h);
+    if (rc != PIC_OK) return rc;
+    *n = h->rb->count[0];
+    return cap < *n ? PIC_ECAPACITY : flags_of(h);
+  }
+  k_read<<<1, 256, 0, h->stream>>>(h->st, instance, h->rb);
+  int rc = read_done(h);
+  if (rc != PIC_OK) return rc;
+  const int32_t count = h->rb->count[species];
   *n = count;
   if (cap < count) return PIC_ECAPACITY;
   const int64_t base = h->seg_off[g];
   const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   const size_t bytes = sizeof(float) * (size_t)count;
   if (count > 0) {
+    cudaError_t e = cudaSuccess;
     if (z && e == cudaSuccess) e = cudaMemcpyAsync(z, h->st.z + base, bytes, kind, h->stream);
     if (vx && e == cudaSuccess) e = cudaMemcpyAsync(vx, h->st.vx + base, bytes, kind, h->stream);
     if (vy && e == cudaSuccess) e = cudaMemcpyAsync(vy, h->st.vy + base, bytes, kind, h->stream);
     if (vz && e == cudaSuccess) e = cudaMemcpyAsync(vz, h->st.vz + base, bytes, kind, h->stream);
     if (id && e == cudaSuccess) e = cudaMemcpyAsync(id, h->st.id + base, bytes, kind, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return cuda_fail(h, e);
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  return check_flags(h);
+  return flags_of(h);
 }
 
 int pic_get_rho_fixed(pic_handle* h, int instance, int64_t* out, int64_t n_nodes) {
@@ -1152,11 +1246,11 @@ int pic_get_rho_fixed(pic_handle* h, int instance, int64_t* out, int64_t n_nodes
   if (n_nodes < nn) return PIC_EINVAL;
   int rc = ensure_field(h);
   if (rc != PIC_OK) return rc;
-  cudaError_t e = cudaMemcpyAsync(out, h->st.rho + h->ic[instance].node_off, sizeof(int64_t) * nn,
-                                  cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  return check_flags(h);
+  k_read_rho<<<1, 512, 0, h->stream>>>(h->st, instance, h->rb);
+  rc = read_done(h);
+  if (rc != PIC_OK) return rc;
+  std::memcpy(out, (const char*)h->rb + kReadNodes, sizeof(int64_t) * nn);
+  return flags_of(h);
 }
 
 int pic_get_field(pic_handle* h, int instance, double* phi, float* E, int64_t n_nodes) {
@@ -1165,17 +1259,14 @@ int pic_get_field(pic_handle* h, int instance, double* phi, float* E, int64_t n_
   if (n_nodes < nn) return PIC_EINVAL;
   int rc = ensure_field(h);
   if (rc != PIC_OK) return rc;
-  const int off = h->ic[instance].node_off;
   // a step computes E only; phi of the current state is solved on request
-  k_phi<<<h->n_inst, kPostThreads, h->field_smem, h->stream>>>(h->st);
-  cudaError_t e = cudaGetLastError();
-  if (phi && e == cudaSuccess)
-    e = cudaMemcpyAsync(phi, h->st.phi + off, sizeof(double) * nn, cudaMemcpyDeviceToHost, h->stream);
-  if (E && e == cudaSuccess)
-    e = cudaMemcpyAsync(E, h->st.E + off, sizeof(float) * nn, cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  return check_flags(h);
+  k_phi<<<1, kPostThreads, h->field_smem, h->stream>>>(h->st, instance, h->rb);
+  rc = read_done(h);
+  if (rc != PIC_OK) return rc;
+  const char* nodes = (const char*)h->rb + kReadNodes + sizeof(double) * nn;
+  if (phi) std::memcpy(phi, nodes, sizeof(double) * nn);
+  if (E) std::memcpy(E, nodes + sizeof(double) * nn, sizeof(float) * nn);
+  return flags_of(h);
 }
 
 int pic_set_profile_period(pic_handle* h, int64_t period) {
@@ -1411,6 +1502,7 @@ int pic_load(pic_handle* h, const void* host_buf, size_t bytes) {
     if (d.step != hd.step) return PIC_EINVAL;
   if (ckpt_bytes(h, counts, hd.has_prof != 0) > bytes) return PIC_EINVAL;
   // validated: from here on the handle takes the checkpoint's state
+  h->counts_known = false;
   if (hd.has_prof) {
     if (!h->st.phi_sum) {          // allocate the sums (overwritten below)
       int rc = pic_set_profile_period(h, 1);
@@ -1510,6 +1602,7 @@ void pic_destroy(pic_handle* h) {
   drop_graph(h);
   free_all(h);
   if (h->stream) cudaStreamSynchronize(h->stream);
+  readback_give(h->rb);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
 }

@@ -111,6 +111,20 @@ struct PostScratch {
   double ke[3][kMaxParts][2];
 };
 
+// What a reading call gets back, written by a kernel into mapped host memory
+// (one launch and one synchronisation, no staged copies); node arrays follow
+// at kReadNodes.
+struct Readback {
+  int err;                 // error bits of all diodes
+  int bad;                 // pic_inject: blocks that saw a z outside [0, L)
+  int count[3];            // live particles of the diode
+  int pad;
+  InstDyn dyn;
+};
+constexpr size_t kReadNodes = 1024;
+constexpr size_t kReadBytes = kReadNodes + (size_t)(kMaxNz + 1) * 20;   // rho, phi (8 B), E
+static_assert(sizeof(Readback) <= kReadNodes && sizeof(InstDyn) % 4 == 0, "layout");
+
 struct Event {              // one ionisation: parent id + both children
   uint32_t parent;
   float z;

@@ -1173,18 +1173,102 @@ __global__ void __launch_bounds__(kPostThreads) k_field(DevState st) {
   field_solve(ic, rho_s, st.E + off, st.phi + off, ws64);
 }
 
-// phi (and E, identically) of the current state from its fixed-point charge,
-// for callers that read the potential; a time step computes E only.
-__global__ void __launch_bounds__(kPostThreads) k_phi(DevState st) {
+// ------------------------------------------------------------------ readback
+// error bits of all diodes into out (all threads call)
+__device__ __forceinline__ void read_errors(const DevState& st, Readback* out) {
+  int e = 0;
+  for (int i = threadIdx.x; i < st.n_inst; i += blockDim.x) e |= st.dyn[i].err;
+  __shared__ int any;
+  if (threadIdx.x == 0) any = 0;
+  __syncthreads();
+  e = (int)__reduce_or_sync(0xffffffffu, (unsigned)e);
+  if ((threadIdx.x & 31) == 0 && e) atomicOr(&any, e);
+  __syncthreads();
+  if (threadIdx.x == 0) out->err = any;
+}
+
+// errors and, for inst >= 0, the diode's record and counts
+__global__ void k_read(DevState st, int inst, Readback* out) {
+  read_errors(st, out);
+  if (inst < 0) return;
+  const int* src = reinterpret_cast<const int*>(st.dyn + inst);
+  int* dst = reinterpret_cast<int*>(&out->dyn);
+  for (int w = threadIdx.x; w < (int)(sizeof(InstDyn) / 4); w += blockDim.x) dst[w] = src[w];
+  if (threadIdx.x < 3) out->count[threadIdx.x] = st.seg_count[3 * inst + threadIdx.x];
+}
+
+// errors and the diode's fixed-point charge
+__global__ void k_read_rho(DevState st, int inst, Readback* out) {
+  const InstConst& ic = st.ic[inst];
+  long long* rho = reinterpret_cast<long long*>(reinterpret_cast<char*>(out) + kReadNodes);
+  for (int j = threadIdx.x; j <= ic.Nz; j += blockDim.x) rho[j] = st.rho[ic.node_off + j];
+  read_errors(st, out);
+}
+
+// phi (and E, identically) of one diode's current state from its fixed-point
+// charge, for callers that read the potential; a time step computes E only.
+__global__ void __launch_bounds__(kPostThreads) k_phi(DevState st, int inst, Readback* out) {
   extern __shared__ __align__(16) unsigned char smem[];
   long long* rho_s = reinterpret_cast<long long*>(smem);
   __shared__ long long ws64[32];
-  const InstConst& ic = st.ic[blockIdx.x];
+  const InstConst& ic = st.ic[inst];
   const int nn = ic.Nz + 1;
   const int off = ic.node_off;
   for (int j = threadIdx.x; j < nn; j += blockDim.x) rho_s[j] = st.rho[off + j];
   __syncthreads();
   field_solve(ic, rho_s, st.E + off, st.phi + off, ws64);
+  double* phi = reinterpret_cast<double*>(reinterpret_cast<char*>(out) + kReadNodes) + nn;
+  float* E = reinterpret_cast<float*>(phi + nn);
+  for (int j = threadIdx.x; j < nn; j += blockDim.x) {
+    phi[j] = st.phi[off + j];
+    E[j] = st.E[off + j];
+  }
+  read_errors(st, out);
+}
+
+// The live particles of segment g into the caller's device arrays (null ones
+// are skipped; nothing is copied if there are more than cap), with the count
+// and the errors: one launch, sized by the host from the capacity, since only
+// the device knows the count.  vec: every array is 16-byte aligned.
+template <typename T>
+__device__ __forceinline__ void copy_out(T* dst, const T* src, int n, int vec) {
+  if (!dst) return;
+  const int i0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  int done = 0;
+  if (vec) {
+    const uint4* s4 = reinterpret_cast<const uint4*>(src);
+    uint4* d4 = reinterpret_cast<uint4*>(dst);
+    const int nq = n >> 2;
+    int i = i0;
+    for (; i + 3 * stride < nq; i += 4 * stride) {
+      const uint4 a = s4[i], b = s4[i + stride], c = s4[i + 2 * stride], d = s4[i + 3 * stride];
+      d4[i] = a;
+      d4[i + stride] = b;
+      d4[i + 2 * stride] = c;
+      d4[i + 3 * stride] = d;
+    }
+    for (; i < nq; i += stride) d4[i] = s4[i];
+    done = nq * 4;
+  }
+  for (int i = done + i0; i < n; i += stride) dst[i] = src[i];
+}
+
+__global__ void __launch_bounds__(256) k_state_copy(DevState st, int g, long long cap, float* z,
+                                                    float* vx, float* vy, float* vz, uint32_t* id,
+                                                    int vec, Readback* out) {
+  const int n = st.seg_count[g];
+  const long long off = st.seg_off[g];
+  if (n <= cap) {
+    copy_out(z, st.z + off, n, vec);
+    copy_out(vx, st.vx + off, n, vec);
+    copy_out(vy, st.vy + off, n, vec);
+    copy_out(vz, st.vz + off, n, vec);
+    copy_out(id, st.id + off, n, vec);
+  }
+  if (blockIdx.x == 0) {
+    read_errors(st, out);
+    if (threadIdx.x == 0) out->count[0] = n;
+  }
 }
 
 // ------------------------------------------------------------------ weights
@@ -1790,20 +1874,62 @@ __global__ void __launch_bounds__(256) k_profile(DevState st) {
   hist_flush(h, Nz, 1LL, st.prof + (long long)sp * st.tn + ic.node_off);
 }
 
-// ------------------------------------------------------------------ helpers
-__global__ void k_fill_ids(uint32_t* id, long long n, uint32_t first) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) id[i] = first + (uint32_t)i;
+// ------------------------------------------------------------------ injection
+// n particles into the free slots from `at` on: ids first, first + 1, ..., z
+// checked against [0, Lf) (bad counts the blocks that saw one outside), and
+// the fields copied from device arrays unless zs is null (they are there
+// already).  One pass, 16 B read and 20 B written per particle.  vec: at and
+// the arrays are 16-byte aligned.
+__global__ void __launch_bounds__(256) k_inject(DevState st, long long at, long long n,
+                                                const float* zs, const float* vxs,
+                                                const float* vys, const float* vzs, uint32_t first,
+                                                float Lf, int vec, int* bad) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  bool out = false;
+  if (vec && 4 * i + 3 < n) {
+    float4 z;
+    if (zs) {
+      z = reinterpret_cast<const float4*>(zs)[i];
+      const float4 a = reinterpret_cast<const float4*>(vxs)[i];
+      const float4 b = reinterpret_cast<const float4*>(vys)[i];
+      const float4 c = reinterpret_cast<const float4*>(vzs)[i];
+      reinterpret_cast<float4*>(st.z + at)[i] = z;
+      reinterpret_cast<float4*>(st.vx + at)[i] = a;
+      reinterpret_cast<float4*>(st.vy + at)[i] = b;
+      reinterpret_cast<float4*>(st.vz + at)[i] = c;
+    } else {
+      z = reinterpret_cast<const float4*>(st.z + at)[i];
+    }
+    const uint32_t d = first + (uint32_t)(4 * i);
+    reinterpret_cast<uint4*>(st.id + at)[i] = make_uint4(d, d + 1u, d + 2u, d + 3u);
+    out = !(z.x >= 0.0f && z.x < Lf && z.y >= 0.0f && z.y < Lf && z.z >= 0.0f && z.z < Lf &&
+            z.w >= 0.0f && z.w < Lf);
+  } else {
+    for (long long k = 4 * i; k < n && k < 4 * i + 4; ++k) {
+      const float z = zs ? zs[k] : st.z[at + k];
+      if (zs) {
+        st.z[at + k] = z;
+        st.vx[at + k] = vxs[k];
+        st.vy[at + k] = vys[k];
+        st.vz[at + k] = vzs[k];
+      }
+      st.id[at + k] = first + (uint32_t)k;
+      out |= !(z >= 0.0f && z < Lf);
+    }
+  }
+  if (__syncthreads_or(out) && threadIdx.x == 0) atomicAdd(bad, 1);
 }
 
-__global__ void k_count_outside(const float* z, long long n, float Lf, int* bad) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  int b = 0;
-  if (i < n) {
-    const float v = z[i];
-    b = !(v >= 0.0f && v < Lf);
+// The particles of a call count only if every z lay inside; bad is zero again
+// for the next call.
+__global__ void k_inject_commit(DevState st, int g, int count, uint32_t next_id, int* bad,
+                                Readback* out) {
+  out->bad = *bad;
+  if (*bad == 0) {
+    st.seg_count[g] = count;
+    st.dyn[g / 3].next_id = next_id;
   }
-  if (__syncthreads_or(b) && threadIdx.x == 0) atomicAdd(bad, 1);
+  *bad = 0;
 }
 
 }  // namespace pic
