@@ -2,7 +2,7 @@
 //
 // A step of a diode with a few tens of thousands of particles is bound by the
 // three dependent kernels and the round trips inside them (17.1 us a step for
-// 22k particles), not by its work.  Here a thread-block cluster (1 to 8
+// 22k particles), not by its work.  Here a thread-block cluster (1 to 16
 // blocks, by how many diodes share the chip) owns a diode and runs n_steps of
 // it: field, constants, counts and tallies stay in shared memory, the
 // particles in L2, and the phases of a step meet at hardware cluster
@@ -23,8 +23,8 @@
 //      summed over the blocks; collisions of the blocks' candidates
 //   C  kinetic energies of the absorbed particles read (last block); the
 //      particles that will fill their slots looked up and read; the field, by
-//      every block for itself, the prefix in its last warp (from
-//      kFusedWarpCells cells on all warps solve it in B)
+//      every block for itself, the prefix in its last warp (in all
+//      of them from kFusedWarpCells cells on)
 //   D  the tallies summed (last block), hole filling and appends (a species
 //      per block, or per part of the block's warps)
 //
@@ -39,11 +39,10 @@ namespace pic {
 namespace cg = cooperative_groups;
 
 constexpr int kFusedWarps = kFusedThreads / 32;
-constexpr int kFusedMaxC = 8;          // portable cluster size
+constexpr int kFusedMaxC = 16;         // blocks per cluster (non-portable above 8)
 constexpr int kFusedCand = 1024;       // candidates listed per block and step
 constexpr int kFusedList = 1024;       // absorbed slots of a species held in shared memory
 constexpr int kFusedWarpList = 32;     // of a warp and species
-constexpr int kFusedWarpCells = 512;   // cells that one warp solves for
 constexpr int kFusedTeamWarps = kFusedWarps - 1;   // warps of phase D's teams
 
 // shared memory: (E_j, dE_j) pairs, E, two histograms, the blocks' and the
@@ -521,9 +520,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
     for (int j = tid; j <= Nz; j += nt) {
       const long long v = hist_node(histI, j, Nz) - hist_node(histE, j, Nz);
       if (warp_field) {
-#pragma unroll
-        for (int b = 0; b < kFusedMaxC; ++b)
-          if (b < C) cl.map_shared_rank(node, b)[rank * mn + j] = v;
+#pragma unroll 2
+        for (int b = 0; b < C; ++b) cl.map_shared_rank(node, b)[rank * mn + j] = v;
       } else {
         node[j] = v;
       }
@@ -535,8 +533,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
     }
     cl.sync();
 
-    // ---- B: absorbed lists, charge (from kFusedWarpCells cells on the whole
-    // field), collisions
+    // ---- B: absorbed lists, charge, collisions
     const int nc = S.ncand, Nem = S.nemit;
     int D[3], start[3];
     {
@@ -560,18 +557,25 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
                                          : st.dead_buf + S.off[sp];
       for (int k = lane; k < n; k += 32) to[start[sp] + k] = k < kFusedWarpList ? near[k] : far[k];
     }
-    for (int j = tid; j <= Nz; j += nt) {
-      long long v = 0;
-#pragma unroll
-      for (int b = 0; b < kFusedMaxC; ++b)
-        if (b < C) v += warp_field ? node[b * mn + j] : cl.map_shared_rank(node, b)[j];
-      rho_s[warp_field ? fused_at(j) : j] = v;
-      if (rank == 0 && it == n_steps - 1) st.rho[ic.node_off + j] = v;
-    }
-    if (!warp_field) {
-      __syncthreads();
-      field_solve(ic, rho_s, E, nullptr, S.ws64);
-      for (int j = tid; j < Nz; j += nt) Es2[j] = make_float2(E[j], E[j + 1] - E[j]);
+    if (warp_field) {
+      for (int j = tid; j <= Nz; j += nt) {
+        long long v = 0;
+#pragma unroll 4
+        for (int b = 0; b < C; ++b) v += node[b * mn + j];
+        rho_s[fused_at(j)] = v;
+        if (rank == 0 && it == n_steps - 1) st.rho[ic.node_off + j] = v;
+      }
+    } else {
+      // a slice of the nodes per block, summed from and written to all of them
+      const int j0 = (int)((long long)(Nz + 1) * rank / C), j1 = (int)((long long)(Nz + 1) * (rank + 1) / C);
+      for (int j = j0 + tid; j < j1; j += nt) {
+        long long v = 0;
+#pragma unroll 4
+        for (int b = 0; b < C; ++b) v += cl.map_shared_rank(node, b)[j];
+#pragma unroll 2
+        for (int b = 0; b < C; ++b) cl.map_shared_rank(rho_s, b)[j] = v;
+        if (it == n_steps - 1) st.rho[ic.node_off + j] = v;
+      }
     }
     if (nc <= kFusedCand) {
       for (int k = nt - 1 - tid; k < nc; k += nt) {
@@ -647,7 +651,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
     if (team < post_n && warp < kFusedWarps - 1 && post_sp == 0 && tm.tid < Nem)
       emitted_electron(ic, tm.tid, step, drawn.x, drawn.y, drawn.z, drawn.w);
     if (Dp > 0) fused_move(st, tm.tid, n_of(post_sp), Dp, off_of(post_sp), dd_post, mv);
-    if (warp_field) {
+    if (!warp_field) {
+      field_solve(ic, rho_s, E, nullptr, S.ws64);
+    } else {
       __syncthreads();                 // the prefix
       const double A = S.fA, B = S.fB;
       for (int j = tid; j <= Nz; j += nt) {
@@ -660,8 +666,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
     cl.sync();
 
     // ---- D: hole filling, appends, tallies
-    if (warp_field)
-      for (int j = tid; j < Nz; j += nt) Es2[j] = make_float2(E[j], E[j + 1] - E[j]);
+    for (int j = tid; j < Nz; j += nt) Es2[j] = make_float2(E[j], E[j + 1] - E[j]);
     if (warp == kFusedWarps - 1) {
       if (rank == last) emit_charge(step + 1, lane, 32);
     } else if (team < post_n) {
@@ -742,9 +747,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
 }
 
 // Which way the next steps run: 1 (the fused kernel) if its estimated time per
-// step is the smaller.  A cluster takes T0 and its diode's particles at the
-// rate of its blocks, the clusters share the SMs; the three kernels take their
-// launches, a part per diode and the particles at the chip's rate.
+// step is the smaller.
 // The fused kernel's histograms hold kHistMaxParticles per block, so it is not
 // taken where `growth` (most particles a diode can gain over the steps) could
 // pass that, nor where the expected candidates come near the size of the three
@@ -772,13 +775,8 @@ __global__ void k_route(DevState st, int C, int sms, long long growth,
   cands = block_sum<float>(cands, wsc);
   if (threadIdx.x == 0) {
     for (int w = 1; w < (int)(blockDim.x >> 5); ++w) longest = fmaxf(longest, wsf[w]);
-    const float t0 = kFusedStepNs + kFusedBlockNs * (float)C + kFusedCellNs * (float)st.max_nodes;
-    const float per = 1.0f / (kFusedRate * (float)C);
-    const float chain = t0 + longest * per;
-    const float work = ((float)st.n_inst * t0 + (float)total * per) * (float)C / (float)sms;
-    const float fused = fmaxf(chain, work);
-    const float three = kThreeStepNs + kThreeDiodeNs * (float)st.n_inst + (float)total / kThreeRate;
-    const bool one = fused < three && 2.0f * cands + 4096.0f < (float)st.cand_cap &&
+    const StepEstimate e = estimate_step(st.n_inst, longest, (float)total, C, sms, st.max_nodes);
+    const bool one = e.fused < e.three && 2.0f * cands + 4096.0f < (float)st.cand_cap &&
                      (long long)longest + growth < (long long)kHistMaxParticles;
     cudaGraphSetConditional(handle, one ? 1u : 0u);
   }

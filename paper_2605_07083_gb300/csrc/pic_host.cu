@@ -102,7 +102,7 @@ struct pic_handle {
   int bstart_len = 0;
   int* inject_flag = nullptr;   // device word: an injected z outside [0, L)
   Readback* rb = nullptr;       // mapped host memory the reading kernels write
-  // live counts and next ids while no step has run since they were known
+  // live counts and next ids as last known; counts_known: no step has run since
   bool counts_known = false;
   std::vector<int32_t> known_count;
   std::vector<uint32_t> known_id;
@@ -306,6 +306,11 @@ int check_flags(pic_handle* h) {
   return rc == PIC_OK ? flags_of(h) : rc;
 }
 
+// a diode's counts after a k_read of it
+void note_counts(pic_handle* h, int instance) {
+  for (int s = 0; s < 3; ++s) h->known_count[3 * instance + s] = h->rb->count[s];
+}
+
 // Device arrays that a kernel may read or write: device or managed memory,
 // aligned to their elements.  Anything else goes through cudaMemcpyAsync,
 // which handles it or refuses it.  *vec: all are 16-byte aligned.
@@ -361,6 +366,8 @@ cudaError_t raise_smem_limits(int device) {
 
     if (e != cudaSuccess) return e;
   }
+  e = cudaFuncSetAttribute((const void*)k_fused, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
   e = sort_prepare(optin);
   if (e == cudaSuccess && device >= 0 && device < 64) done[device] = true;
   return e;
@@ -639,12 +646,13 @@ cudaError_t enqueue_fused(pic_handle* h, int n) {
 }
 
 // Blocks per diode of k_fused: as many as let all clusters be resident at
-// once, a power of two up to the portable cluster size; 0 where a block does
-// not fit (its shared memory grows with the cells).
+// once, a power of two up to 16 (a cluster of 16, which has to be allowed,
+// takes 9.8 us for 22k particles and 15.4 for 135k, one of 8 10.4 and 18.4); 0
+// where a block does not fit (its shared memory grows with the cells).
 void set_fused_shape(pic_handle* h) {
   h->fused_c = 0;
   h->fused_smem = fused_smem_bytes(h->max_nodes);
-  for (int c = 8; c >= 1 && h->fused_c == 0; c /= 2) {
+  for (int c = 16; c >= 1 && h->fused_c == 0; c /= 2) {
     if (c > 1 && h->n_inst * c > h->sm_count) continue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(h->n_inst * c));
@@ -664,10 +672,22 @@ void set_fused_shape(pic_handle* h) {
   cudaGetLastError();                  // a shape that does not fit is no error
 }
 
-// k_fused takes neither sorts nor profile samples, and has no bulk-copy wait
-// to give up on
+// Step graphs let the device choose k_fused?  It takes neither sorts nor
+// profile samples, and has no bulk-copy wait to give up on.  The choice costs
+// ~15 us per kRouteSteps steps (a kernel and a conditional node), so it is not
+// offered where the last counts the host knows make k_fused take twice the
+// time of the three kernels.
 bool fused_allowed(const pic_handle* h) {
-  return h->fused_c > 0 && h->sort_period <= 0 && h->st.prof_period <= 0 &&
+  long long total = 0;
+  int longest = 0;
+  for (int i = 0; i < h->n_inst; ++i) {
+    const int n = h->known_count[3 * i] + h->known_count[3 * i + 1] + h->known_count[3 * i + 2];
+    total += n;
+    longest = std::max(longest, n);
+  }
+  const StepEstimate e = estimate_step(h->n_inst, (float)longest, (float)total,
+                                       std::max(1, h->fused_c), h->sm_count, h->max_nodes);
+  return h->fused_c > 0 && e.fused < 2.0f * e.three && h->sort_period <= 0 && h->st.prof_period <= 0 &&
          h->st.wait_limit == kWaitLimit;
 }
 
@@ -1018,7 +1038,8 @@ int pic_inject(pic_handle* h, int instance, int species, int64_t n, const float*
     int rc = read_done(h);
     if (rc != PIC_OK) return rc;
   }
-  const int32_t count = h->counts_known ? h->known_count[g] : h->rb->count[species];
+  if (!h->counts_known) note_counts(h, instance);
+  const int32_t count = h->known_count[g];
   const uint32_t next_id = h->counts_known ? h->known_id[instance] : h->rb->dyn.next_id;
   if ((int64_t)count + n > h->seg_cap[g]) return PIC_ECAPACITY;
   // the particles go into the free slots after the live ones and their z
@@ -1046,10 +1067,8 @@ int pic_inject(pic_handle* h, int instance, int species, int64_t n, const float*
   int rc = read_done(h);
   if (rc != PIC_OK) return rc;
   if (h->rb->bad) return PIC_EINVAL;
-  if (h->counts_known) {
-    h->known_count[g] = newc;
-    h->known_id[instance] = nid;
-  }
+  h->known_count[g] = newc;
+  h->known_id[instance] = nid;
   h->dirty = true;
   return PIC_OK;
 }
@@ -1198,6 +1217,7 @@ int pic_diagnostics(pic_handle* h, int instance, pic_diag* out) {
   k_read<<<1, 256, 0, h->stream>>>(h->st, instance, h->rb);
   int rc = read_done(h);
   if (rc != PIC_OK) return rc;
+  note_counts(h, instance);
   fill_diag(h, instance, h->rb->dyn, h->rb->count, out);
   return flags_of(h);
 }
@@ -1502,7 +1522,9 @@ int pic_load(pic_handle* h, const void* host_buf, size_t bytes) {
     if (d.step != hd.step) return PIC_EINVAL;
   if (ckpt_bytes(h, counts, hd.has_prof != 0) > bytes) return PIC_EINVAL;
   // validated: from here on the handle takes the checkpoint's state
-  h->counts_known = false;
+  h->counts_known = true;
+  h->known_count = counts;
+  for (int i = 0; i < h->n_inst; ++i) h->known_id[i] = dyn[i].next_id;
   if (hd.has_prof) {
     if (!h->st.phi_sum) {          // allocate the sums (overwritten below)
       int rc = pic_set_profile_period(h, 1);

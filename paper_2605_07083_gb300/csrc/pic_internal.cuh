@@ -32,13 +32,27 @@ enum ErrBit : int32_t { ERR_CAPACITY = 1 << 3, ERR_TIMEOUT = 1 << 4, ERR_ENERGYC
 
 constexpr int kFusedThreads = 512;      // threads per block of k_fused
 constexpr int kFusedMinSteps = 8;      // shortest graph that lets k_route choose
-// k_route's estimate of a step's time, ns: the fused kernel's fixed part, per
-// block of the cluster and per cell, and its particles per ns and block; the
-// three kernels' fixed part, per diode, and particles per ns (fits to the
-// measured steps of 1 to 512 diodes of 128 to 2000 cells)
-constexpr float kFusedStepNs = 7700.0f, kFusedBlockNs = 40.0f, kFusedCellNs = 3.5f;
-constexpr float kFusedRate = 1.8f;
-constexpr float kThreeStepNs = 16000.0f, kThreeDiodeNs = 95.0f, kThreeRate = 270.0f;
+// Estimates of a step's time, ns, by the fused kernel with C blocks per diode
+// and by the three kernels (fits to the measured steps of 1 to 512 diodes of
+// 128 to 2000 cells).  Fused: a cluster takes a fixed time, more per cell and
+// where all warps solve the field, and its diode's particles at the rate of
+// its blocks (2.05 per ns and block, 1.4 in a cluster of 16); the clusters
+// share the SMs.  Three kernels: launches and round trips, a part per diode,
+// the particles at the chip's rate.
+constexpr int kFusedWarpCells = 512;   // cells that one warp of k_fused solves for
+struct StepEstimate { float fused, three; };
+__host__ __device__ inline StepEstimate estimate_step(int n_inst, float longest, float total, int C,
+                                                      int sms, int max_nodes) {
+  const int cells = max_nodes < kFusedWarpCells ? max_nodes : kFusedWarpCells;
+  const float t0 = 8000.0f + 3.5f * (float)cells + (max_nodes > kFusedWarpCells + 1 ? 3500.0f : 0.0f);
+  const float per = 1.0f / ((2.1f - 0.045f * (float)C) * (float)C);
+  const float chain = t0 + longest * per;
+  const float work = ((float)n_inst * t0 + total * per) * (float)C / (float)sms;
+  StepEstimate e;
+  e.fused = chain > work ? chain : work;
+  e.three = 16000.0f + 95.0f * (float)n_inst + total / 270.0f;
+  return e;
+}
 
 // Per-instance constants, derived on the host in FP64 and stored once.
 struct InstConst {

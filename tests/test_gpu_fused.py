@@ -1,7 +1,7 @@
 """Whole steps of small diodes in one kernel (chosen on the device inside the
 step graphs) against the three kernels launched one by one: array order,
 charge, field, tallies (the FP64 energies too) bit for bit.  The diode counts
-give clusters of 8, 4, 2 and 1 blocks; the cases reach partial quads, an empty
+give clusters of 16 to 1 blocks; the cases reach partial quads, an empty
 species, replenishment, ionisation, more candidates than a block lists, more
 absorbed particles than a warp's lanes and than the staged list, and growth
 past the point where the choice changes.  GPU."""
@@ -31,6 +31,8 @@ def _diodes(n_inst, kind):
         elif kind == "hot":                # most particles leave within a few steps
             p.update(n_gas=0.0, T_e0_eV=1e5, dt=1e-11, replenish=1, Nz=127 + i)
             n_emit, n_pairs = 700, 9000
+        elif kind == "wide":               # more cells than one warp solves for
+            p.update(Nz=(600, 1999, 513)[i % 3], dt=2e-13)
         elif kind == "emission":           # 3000 electrons a step: outgrows the choice
             p.update(gamma_emit=p["gamma_emit"] * 1000.0, capacity=(1 << 18, 65536, 65536))
         ps.append(p)
@@ -42,7 +44,7 @@ def _diodes(n_inst, kind):
 @pytest.mark.parametrize("n_inst,kind,steps", [
     (1, "plain", 200), (1, "empty", 70), (1, "dense", 40), (1, "hot", 12), (1, "emission", 130),
     (20, "plain", 33), (39, "dense", 9), (39, "hot", 9), (100, "plain", 17), (100, "dense", 9),
-    (170, "plain", 9),
+    (170, "plain", 9), (1, "wide", 70), (5, "wide", 40), (100, "wide", 9),
 ])
 def test_fused_steps_match_the_three_kernels(n_inst, kind, steps):
     torch = pytest.importorskip("torch")
