@@ -23,8 +23,7 @@ constexpr int oW1 = 0, ob1 = oW1 + H * IN, oW2 = ob1 + H, ob2 = oW2 + H * H, oW3
               ob3 = oW3 + H * H, oW4 = ob3 + H, ob4 = oW4 + OUT * H, NP = ob4 + OUT;
 static_assert(NP == PIC_MLP_PARAMS, "parameter count");
 
-// The block works on a tile of TS samples (8, 16, 32; 128 for prediction) with
-// 16 warps.  Every
+// The block works on a tile of TS samples (8, 16 or 32) with 16 warps.  Every
 // activation array is [unit][sample] with rows of TS + 4 floats: the samples
 // of a unit are consecutive (128-bit loads of four), and rows start 4 banks
 // apart (mod 8 groups of 4), so lanes on neighbouring units never collide.
@@ -46,7 +45,7 @@ constexpr int kSms = 152;                    // tiles are kept to one wave while
 template <int TS>
 struct Tile {
   static constexpr int kRow = TS + 4;        // floats per row of an activation array
-  static constexpr int kSpw = TS > 32 ? 8 : 4;   // samples per warp
+  static constexpr int kSpw = 4;             // samples per warp
   static constexpr int kSg = TS / kSpw;      // groups of that many
   static constexpr int kSplit = kWarps / kSg;    // warps that share a group's contraction
 };
@@ -101,52 +100,88 @@ __device__ __forceinline__ float gelu(float x, float& slope) {
 }
 
 // 128 x 128 bfloat16 W (row-major [j][k]) into shared memory as [k][j]: a
-// thread takes two rows' next eight columns and writes eight (j, j + 1) words
-__device__ __forceinline__ void load_transposed(const __nv_bfloat16* __restrict__ W,
-                                                __nv_bfloat16 (*wt)[kWRow]) {
-  const unsigned short* src = reinterpret_cast<const unsigned short*>(W);
-  unsigned* dst = reinterpret_cast<unsigned*>(wt);
-  const bool wide = (reinterpret_cast<unsigned long long>(W) & 15ull) == 0ull;
-#pragma unroll
-  for (int r = 0; r < (H / 2) * (H / 8) / kThr; ++r) {
-    const int t = r * kThr + (int)threadIdx.x;
-    const int jp = t & (H / 2 - 1), k0 = (t >> 6) * 8;
-    const unsigned short* p0 = src + (2 * jp) * H + k0;
+// thread takes two rows' next eight columns and writes eight (j, j + 1) words.
+// Fetch and store are apart so that the loads of both matrices and of the
+// small arrays are in flight together.
+constexpr int kTasks = (H / 2) * (H / 8);      // (row pair, eight columns)
+
+__device__ __forceinline__ void fetch_rows(const __nv_bfloat16* __restrict__ W, int t, uint4& u,
+                                           uint4& v) {
+  const unsigned short* p0 =
+      reinterpret_cast<const unsigned short*>(W) + (2 * (t & (H / 2 - 1))) * H + (t >> 6) * 8;
+  if ((reinterpret_cast<unsigned long long>(W) & 15ull) == 0ull) {
+    u = *reinterpret_cast<const uint4*>(p0);
+    v = *reinterpret_cast<const uint4*>(p0 + H);
+  } else {
     unsigned x[4], y[4];
-    if (wide) {
-      const uint4 u = *reinterpret_cast<const uint4*>(p0);
-      const uint4 v = *reinterpret_cast<const uint4*>(p0 + H);
-      x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
-      y[0] = v.x; y[1] = v.y; y[2] = v.z; y[3] = v.w;
-    } else {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        x[q] = (unsigned)p0[2 * q] | ((unsigned)p0[2 * q + 1] << 16);
-        y[q] = (unsigned)p0[H + 2 * q] | ((unsigned)p0[H + 2 * q + 1] << 16);
-      }
-    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      dst[(k0 + 2 * q) * (kWRow / 2) + jp] = __byte_perm(x[q], y[q], 0x5410);
-      dst[(k0 + 2 * q + 1) * (kWRow / 2) + jp] = __byte_perm(x[q], y[q], 0x7632);
+      x[q] = (unsigned)p0[2 * q] | ((unsigned)p0[2 * q + 1] << 16);
+      y[q] = (unsigned)p0[H + 2 * q] | ((unsigned)p0[H + 2 * q + 1] << 16);
     }
+    u = make_uint4(x[0], x[1], x[2], x[3]);
+    v = make_uint4(y[0], y[1], y[2], y[3]);
   }
 }
 
-template <int TS>
-__device__ __forceinline__ void load_weights(Smem<TS>& S, const float* __restrict__ master,
-                                             const __nv_bfloat16* __restrict__ w) {
-  const int tid = threadIdx.x;
-  load_transposed(w + oW2, S.w2t);
-  load_transposed(w + oW3, S.w3t);
-  for (int i = tid; i < H * IN; i += kThr) S.w1t[i % IN][i / IN] = __bfloat162float(w[oW1 + i]);
-  for (int i = tid; i < OUT * H; i += kThr) S.w4[i / H][i % H] = __bfloat162float(w[oW4 + i]);
-  if (tid < H) {
-    S.b1[tid] = master[ob1 + tid];
-    S.b2[tid] = master[ob2 + tid];
-    S.b3[tid] = master[ob3 + tid];
+__device__ __forceinline__ void store_rows(__nv_bfloat16 (*wt)[kWRow], int t, const uint4& u,
+                                           const uint4& v) {
+  unsigned* dst = reinterpret_cast<unsigned*>(wt);
+  const int jp = t & (H / 2 - 1), k0 = (t >> 6) * 8;
+  const unsigned x[4] = {u.x, u.y, u.z, u.w}, y[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    dst[(k0 + 2 * q) * (kWRow / 2) + jp] = __byte_perm(x[q], y[q], 0x5410);
+    dst[(k0 + 2 * q + 1) * (kWRow / 2) + jp] = __byte_perm(x[q], y[q], 0x7632);
   }
-  if (tid < OUT) S.b4[tid] = master[ob4 + tid];
+}
+
+__device__ __forceinline__ void load_transposed(const __nv_bfloat16* __restrict__ W,
+                                                __nv_bfloat16 (*wt)[kWRow], int threads) {
+#pragma unroll 2
+  for (int t = threadIdx.x; t < kTasks; t += threads) {
+    uint4 u, v;
+    fetch_rows(W, t, u, v);
+    store_rows(wt, t, u, v);
+  }
+}
+
+// the weights, biases and the tile's inputs; the caller's first barrier follows
+template <int TS>
+__device__ __forceinline__ void load_tile(Smem<TS>& S, const float* __restrict__ master,
+                                          const __nv_bfloat16* __restrict__ w,
+                                          const float* __restrict__ x, long long s0, int ns) {
+  static_assert(kTasks == 2 * kThr && H * IN <= 2 * kThr && OUT * H == kThr && 3 * H <= kThr &&
+                    TS * IN <= kThr, "loads per thread");
+  const int tid = threadIdx.x;
+  uint4 u2[2], v2[2], u3[2], v3[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    fetch_rows(w + oW2, tid + r * kThr, u2[r], v2[r]);
+    fetch_rows(w + oW3, tid + r * kThr, u3[r], v3[r]);
+  }
+  const int xs = tid / IN, xk = tid - xs * IN;
+  const float xv = tid < TS * IN && xs < ns ? x[s0 * IN + tid] : 0.0f;
+  const __nv_bfloat16 wa = w[oW1 + tid];
+  const bool more = tid + kThr < H * IN;
+  const __nv_bfloat16 wb = more ? w[oW1 + tid + kThr] : wa;
+  const __nv_bfloat16 wo = w[oW4 + tid];
+  const int bl = tid / H, bj = tid % H;        // bias of hidden layer bl
+  const float bv = bl < 3 ? master[(bl == 0 ? ob1 : bl == 1 ? ob2 : ob3) + bj]
+                          : (bj < OUT ? master[ob4 + bj] : 0.0f);
+  if (tid < TS * IN) S.a0[xk][xs] = xv;
+  S.w1t[tid % IN][tid / IN] = __bfloat162float(wa);
+  if (more) S.w1t[(tid + kThr) % IN][(tid + kThr) / IN] = __bfloat162float(wb);
+  S.w4[tid / H][tid % H] = __bfloat162float(wo);
+  if (bl == 0) S.b1[bj] = bv;
+  else if (bl == 1) S.b2[bj] = bv;
+  else if (bl == 2) S.b3[bj] = bv;
+  else if (bj < OUT) S.b4[bj] = bv;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    store_rows(S.w2t, tid + r * kThr, u2[r], v2[r]);
+    store_rows(S.w3t, tid + r * kThr, u3[r], v3[r]);
+  }
 }
 
 // acc[r][p] += over this warp's part of the contraction index c of
@@ -353,20 +388,15 @@ __device__ __forceinline__ void weight_grad(const float (*d)[Tile<TS>::kRow],
   }
 }
 
-// inputs of the tile, layers 1 to 3 and the output partial sums; y of
+// layers 1 to 3 and the output partial sums of a loaded tile; y of
 // output o and sample s is then y_of(S, o, s)
 template <int TS, bool kGrad>
-__device__ __forceinline__ void forward_tile(Smem<TS>& S, SmemGrad<TS>* G,
-                                             const float* __restrict__ x, long long s0, int ns) {
+__device__ __forceinline__ void forward_tile(Smem<TS>& S, SmemGrad<TS>* G, int ns) {
   // training computes whole tiles (samples past the batch read zeros and get
   // delta 0), prediction only the groups of four that hold samples
   const int live = kGrad ? TS : (ns + 3) & ~3;
   const int tid = threadIdx.x;
-  for (int i = tid; i < TS * IN; i += kThr) {
-    const int s = i / IN, k = i - s * IN;
-    S.a0[k][s] = s < ns ? x[(s0 + s) * IN + k] : 0.0f;
-  }
-  __syncthreads();
+  __syncthreads();                     // load_tile
   for (int e = tid; e < H * (live / 4); e += kThr) {
     const int j = e % H, s = 4 * (e / H);
     float z[4];
@@ -405,26 +435,151 @@ __device__ __forceinline__ float y_of(const Smem<TS>& S, int o, int s) {
   return y;
 }
 
-// Prediction: the blocks stride over the tiles of `per` <= TS samples, with
-// the weights kept
+// Prediction of up to a wave of tiles: one block per tile
 template <int TS>
 __global__ void __launch_bounds__(kThr) k_mlp_forward(const float* __restrict__ master,
                                                       const __nv_bfloat16* __restrict__ w,
                                                       const float* __restrict__ x, long long batch,
-                                                      int per, float* __restrict__ y) {
+                                                      float* __restrict__ y) {
   extern __shared__ __align__(16) unsigned char raw[];
   Smem<TS>& S = *reinterpret_cast<Smem<TS>*>(raw);
-  load_weights<TS>(S, master, w);
-  const long long tiles = (batch + per - 1) / per;
-  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const long long s0 = t * per;
-    const int ns = (int)min((long long)per, batch - s0);
-    forward_tile<TS, false>(S, nullptr, x, s0, ns);
-    for (int i = threadIdx.x; i < TS * OUT; i += kThr) {
-      const int s = i / OUT, o = i - s * OUT;
-      if (s < ns) y[(s0 + s) * OUT + o] = y_of<TS>(S, o, s);
+  const long long s0 = (long long)blockIdx.x * TS;
+  const int ns = (int)min((long long)TS, batch - s0);
+  load_tile<TS>(S, master, w, x, s0, ns);
+  forward_tile<TS, false>(S, nullptr, ns);
+  for (int i = threadIdx.x; i < TS * OUT; i += kThr) {
+    const int s = i / OUT, o = i - s * OUT;
+    if (s < ns) y[(s0 + s) * OUT + o] = y_of<TS>(S, o, s);
+  }
+}
+
+// Prediction of large batches: the weights stay in shared memory, and a warp
+// takes eight samples at a time through all layers on its own, so no block
+// barrier ties the warps' FMA phases and erf phases together.  What bounds it:
+// the FMA pipe in the products (16 fma.rn.f32x2 to 8 conversions and 3 shared
+// loads) and issue in the erf, 51 % and 58 % busy over the kernel.  41216
+// samples take 82 us (84 with block tiles of 128 samples, 287 with one thread
+// per unit).  A lane has units 4 l ... 4 l + 3 of all eight samples; the
+// warp's activations are [unit][sample], eight floats a row and four floats
+// of padding every four rows, so that a lane's rows start on banks of their
+// own.
+constexpr int kWideSamples = 8, kWideMaxWarps = 20;
+struct WideSmem {
+  __nv_bfloat16 w2t[H][kWRow], w3t[H][kWRow];
+  float w1t[IN][H], w4[OUT][H];
+  float b1[H], b2[H], b3[H], b4[OUT];
+};
+constexpr int kWideBuf = H * kWideSamples + (H / 4) * 4 + IN * kWideSamples;   // floats per warp
+__device__ __forceinline__ int wide_at(int unit) { return unit * kWideSamples + (unit >> 2) * 4; }
+
+// acc (samples 2 p, 2 p + 1 of unit 4 lane + r) -> activations
+__device__ __forceinline__ void wide_activate(const f2 (&acc)[4][4], float* buf, int lane) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    float a[8], unused;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      a[2 * p] = gelu<false>(lo2(acc[r][p]), unused);
+      a[2 * p + 1] = gelu<false>(hi2(acc[r][p]), unused);
     }
-    // the next tile's barriers come before anything read here is rewritten
+    float4* row = reinterpret_cast<float4*>(buf + wide_at(4 * lane + r));
+    row[0] = make_float4(a[0], a[1], a[2], a[3]);
+    row[1] = make_float4(a[4], a[5], a[6], a[7]);
+  }
+}
+
+__device__ __forceinline__ void wide_layer(const __nv_bfloat16 (*wt)[kWRow], const float* b,
+                                           float* buf, int lane) {
+  f2 acc[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int p = 0; p < 4; ++p) acc[r][p] = pack2(b[4 * lane + r], b[4 * lane + r]);
+#pragma unroll 4
+  for (int c = 0; c < H; ++c) {
+    const uint2 wv = *reinterpret_cast<const uint2*>(&wt[c][4 * lane]);
+    const ulonglong2* row = reinterpret_cast<const ulonglong2*>(buf + wide_at(c));
+    const ulonglong2 a0 = row[0], a1 = row[1];
+    const f2 d[4] = {dup_lo(wv.x), dup_hi(wv.x), dup_lo(wv.y), dup_hi(wv.y)};
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      acc[r][0] = fma2(d[r], a0.x, acc[r][0]);
+      acc[r][1] = fma2(d[r], a0.y, acc[r][1]);
+      acc[r][2] = fma2(d[r], a1.x, acc[r][2]);
+      acc[r][3] = fma2(d[r], a1.y, acc[r][3]);
+    }
+  }
+  __syncwarp();                        // every lane has read the layer below
+  wide_activate(acc, buf, lane);
+  __syncwarp();
+}
+
+__global__ void __launch_bounds__(32 * kWideMaxWarps, 1)
+    k_mlp_forward_wide(const float* __restrict__ master, const __nv_bfloat16* __restrict__ w,
+                       const float* __restrict__ x, long long batch, float* __restrict__ y) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  WideSmem& S = *reinterpret_cast<WideSmem*>(raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = (int)(blockDim.x >> 5);
+  float* buf = reinterpret_cast<float*>(raw + sizeof(WideSmem)) + (size_t)warp * kWideBuf;
+  float* xs = buf + H * kWideSamples + (H / 4) * 4;        // [IN][samples]
+  load_transposed(w + oW2, S.w2t, (int)blockDim.x);
+  load_transposed(w + oW3, S.w3t, (int)blockDim.x);
+  for (int i = tid; i < H * IN; i += blockDim.x) S.w1t[i % IN][i / IN] = __bfloat162float(w[oW1 + i]);
+  for (int i = tid; i < OUT * H; i += blockDim.x) S.w4[i / H][i % H] = __bfloat162float(w[oW4 + i]);
+  for (int i = tid; i < H; i += blockDim.x) {
+    S.b1[i] = master[ob1 + i];
+    S.b2[i] = master[ob2 + i];
+    S.b3[i] = master[ob3 + i];
+  }
+  if (tid < OUT) S.b4[tid] = master[ob4 + tid];
+  __syncthreads();
+  const long long groups = (batch + kWideSamples - 1) / kWideSamples;
+  // consecutive groups to the same warp number of all blocks: every SM gets
+  // its share of the last round
+  for (long long g = (long long)warp * gridDim.x + blockIdx.x; g < groups;
+       g += (long long)warps * gridDim.x) {
+    const long long s0 = g * kWideSamples;
+    const int ns = (int)min((long long)kWideSamples, batch - s0);
+    for (int i = lane; i < IN * kWideSamples; i += 32) {
+      const int s = i / IN, k = i - s * IN;
+      xs[k * kWideSamples + s] = s < ns ? x[(s0 + s) * IN + k] : 0.0f;
+    }
+    __syncwarp();
+    {
+      f2 acc[4][4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int p = 0; p < 4; ++p) acc[r][p] = pack2(S.b1[4 * lane + r], S.b1[4 * lane + r]);
+#pragma unroll
+      for (int k = 0; k < IN; ++k) {
+        const ulonglong2* row = reinterpret_cast<const ulonglong2*>(xs + k * kWideSamples);
+        const ulonglong2 a0 = row[0], a1 = row[1];
+        const float4 wv = *reinterpret_cast<const float4*>(&S.w1t[k][4 * lane]);
+        const float ws[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const f2 d = pack2(ws[r], ws[r]);
+          acc[r][0] = fma2(d, a0.x, acc[r][0]);
+          acc[r][1] = fma2(d, a0.y, acc[r][1]);
+          acc[r][2] = fma2(d, a1.x, acc[r][2]);
+          acc[r][3] = fma2(d, a1.y, acc[r][3]);
+        }
+      }
+      wide_activate(acc, buf, lane);
+    }
+    __syncwarp();
+    wide_layer(S.w2t, S.b2, buf, lane);
+    wide_layer(S.w3t, S.b3, buf, lane);
+    // output o of sample s by lane 8 o + s
+    {
+      const int s = lane & 7, o = lane >> 3;
+      float acc = S.b4[o];
+#pragma unroll 8
+      for (int k = 0; k < H; ++k) acc = fmaf(S.w4[o][k], buf[wide_at(k) + s], acc);
+      if (s < ns) y[(s0 + s) * OUT + o] = acc;
+    }
+    __syncwarp();                      // the buffer is reused
   }
 }
 
@@ -443,8 +598,8 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_fwd_bwd(const float* __restrict
   const int tid = threadIdx.x;
   const long long s0 = (long long)blockIdx.x * TS;
   const int ns = (int)min((long long)TS, batch - s0);
-  load_weights<TS>(S, master, w);
-  forward_tile<TS, true>(S, &G, x, s0, ns);
+  load_tile<TS>(S, master, w, x, s0, ns);
+  forward_tile<TS, true>(S, &G, ns);
   // d(loss)/dy and the squared errors
   {
     float e2 = 0.0f;
@@ -511,7 +666,17 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_fwd_bwd(const float* __restrict
   for (int i = tid; i < H * (IN + 1); i += kThr) {
     const int j = i % H, k = i / H;
     float gw = 0.0f;
-    for (int s = 0; s < TS; ++s) gw = k < IN ? fmaf(G.g1[j][s], S.a0[k < IN ? k : 0][s], gw) : gw + G.g1[j][s];
+#pragma unroll
+    for (int s = 0; s < TS; s += 4) {
+      const float4 d = *reinterpret_cast<const float4*>(&G.g1[j][s]);
+      if (k < IN) {
+        const float4 a = *reinterpret_cast<const float4*>(&S.a0[k][s]);
+        gw = fmaf(d.x, a.x, gw); gw = fmaf(d.y, a.y, gw);
+        gw = fmaf(d.z, a.z, gw); gw = fmaf(d.w, a.w, gw);
+      } else {
+        gw += d.x; gw += d.y; gw += d.z; gw += d.w;
+      }
+    }
     if (k < IN) g[oW1 + j * IN + k] = gw;
     else g[ob1 + j] = gw;
   }
@@ -528,6 +693,9 @@ __global__ void k_mlp_reduce_adam(const float* __restrict__ part, const float* _
                                   float* __restrict__ v, float lr, float beta1, float beta2,
                                   float eps, float bc1, float bc2, int do_adam) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  // launched while the tiles still run (launch_reduce): everything below reads
+  // what they, or launches before them, wrote
+  cudaGridDependencySynchronize();
   if (p == 0 && loss) {
     float L = 0.0f;
     for (int b = 0; b < n_part; ++b) L += lpart[b];
@@ -591,14 +759,40 @@ cudaError_t grad_limit() {
                               (int)(sizeof(Smem<TS>) + sizeof(SmemGrad<TS>)));
 }
 
+constexpr size_t wide_smem(int warps) {
+  return sizeof(WideSmem) + (size_t)warps * kWideBuf * sizeof(float);
+}
+
 bool prepare_kernels() {
   static bool done = false;
   if (!done)
     done = forward_limit<8>() == cudaSuccess && forward_limit<16>() == cudaSuccess &&
-           forward_limit<32>() == cudaSuccess && forward_limit<128>() == cudaSuccess &&
+           forward_limit<32>() == cudaSuccess &&
+           cudaFuncSetAttribute(k_mlp_forward_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)wide_smem(kWideMaxWarps)) == cudaSuccess &&
            grad_limit<8>() == cudaSuccess && grad_limit<16>() == cudaSuccess &&
            grad_limit<32>() == cudaSuccess;
   return done;
+}
+
+// The reduction's launch overlaps the end of the tiles (programmatic stream
+// serialisation): its blocks wait for them to finish.
+cudaError_t launch_reduce(const float* part, const float* lpart, int n_part, long long batch,
+                          float* grad, float* loss, float* master, uint16_t* w, float* m, float* v,
+                          float lr, float beta1, float beta2, float eps, float bc1, float bc2,
+                          int do_adam, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((NP + kRedThreads - 1) / kRedThreads);
+  cfg.blockDim = dim3(kRedThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_mlp_reduce_adam, part, lpart, n_part, batch, grad, loss, master,
+                            reinterpret_cast<__nv_bfloat16*>(w), m, v, lr, beta1, beta2, eps, bc1,
+                            bc2, do_adam);
 }
 
 template <int TS>
@@ -625,17 +819,32 @@ int launch_fwd_bwd(const float* master, const uint16_t* w, const float* x, const
   return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
 }
 
-// One block per SM.  Tiles are cut to whole rounds of them: 41216 samples are
-// three rounds of 92 instead of two and a bit of 128.
 template <int TS>
 void launch_predict(const float* master, const uint16_t* w, const float* x, long long batch,
                     float* y, cudaStream_t s) {
-  const long long rounds = (batch + (long long)kSms * TS - 1) / ((long long)kSms * TS);
-  const long long share = (batch + rounds * kSms - 1) / (rounds * kSms);
-  const int per = TS > 32 ? (int)((share + 3) / 4 * 4) : TS;
-  const long long tiles = (batch + per - 1) / per;
-  k_mlp_forward<TS><<<(unsigned)(tiles < kSms ? tiles : kSms), kThr, sizeof(Smem<TS>), s>>>(
-      master, reinterpret_cast<const __nv_bfloat16*>(w), x, batch, per, y);
+  k_mlp_forward<TS><<<(unsigned)((batch + TS - 1) / TS), kThr, sizeof(Smem<TS>), s>>>(
+      master, reinterpret_cast<const __nv_bfloat16*>(w), x, batch, y);
+}
+
+// One block per SM, of the 12, 16 or 20 warps that leave the fewest idle in
+// the last round (41216 samples: 34 groups per SM are three rounds of 12; two
+// rounds of 17 took 88 us instead of 82: the FMA pipe is no fuller, and the
+// warps' registers spill).
+void launch_predict_wide(const float* master, const uint16_t* w, const float* x, long long batch,
+                         float* y, cudaStream_t s) {
+  const long long groups = (batch + kWideSamples - 1) / kWideSamples;
+  const long long per_sm = (groups + kSms - 1) / kSms;
+  int warps = 16;
+  long long best = -1;
+  for (int n : {16, 20, 12}) {
+    const long long slots = (per_sm + n - 1) / n * n;
+    if (best < 0 || slots < best) {
+      best = slots;
+      warps = n;
+    }
+  }
+  k_mlp_forward_wide<<<kSms, 32 * warps, wide_smem(warps), s>>>(
+      master, reinterpret_cast<const __nv_bfloat16*>(w), x, batch, y);
 }
 
 int launch_forward(const float* master, const uint16_t* w, const float* x, long long batch,
@@ -645,7 +854,7 @@ int launch_forward(const float* master, const uint16_t* w, const float* x, long 
   if (ts == 8) launch_predict<8>(master, w, x, batch, y, s);
   else if (ts == 16) launch_predict<16>(master, w, x, batch, y, s);
   else if (batch <= 32ll * kSms) launch_predict<32>(master, w, x, batch, y, s);
-  else launch_predict<128>(master, w, x, batch, y, s);
+  else launch_predict_wide(master, w, x, batch, y, s);
   return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
 }
 
@@ -682,10 +891,10 @@ int pic_mlp_grad(const float* master, const uint16_t* w_bf16, const float* x, co
   int rc = launch_fwd_bwd(master, w_bf16, x, t, batch, scratch, scratch_bytes,
                           (cudaStream_t)stream, &nblk);
   if (rc != PIC_OK) return rc;
-  k_mlp_reduce_adam<<<(NP + kRedThreads - 1) / kRedThreads, kRedThreads, 0, (cudaStream_t)stream>>>(
-      scratch, scratch + (size_t)nblk * NP, nblk, batch, grad, loss, nullptr, nullptr, nullptr,
-      nullptr, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f, 0);
-  return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
+  const cudaError_t e = launch_reduce(scratch, scratch + (size_t)nblk * NP, nblk, batch, grad, loss,
+                                      nullptr, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, 0.f, 1.f,
+                                      1.f, 0, (cudaStream_t)stream);
+  return e == cudaSuccess ? PIC_OK : PIC_ECUDA;
 }
 
 int pic_mlp_train_step(float* master, uint16_t* w_bf16, float* adam_m, float* adam_v,
@@ -699,11 +908,10 @@ int pic_mlp_train_step(float* master, uint16_t* w_bf16, float* adam_m, float* ad
                           (cudaStream_t)stream, &nblk);
   if (rc != PIC_OK) return rc;
   const float bc1 = 1.0f - powf(beta1, (float)step), bc2 = 1.0f - powf(beta2, (float)step);
-  k_mlp_reduce_adam<<<(NP + kRedThreads - 1) / kRedThreads, kRedThreads, 0, (cudaStream_t)stream>>>(
-      scratch, scratch + (size_t)nblk * NP, nblk, batch, nullptr, loss, master,
-      reinterpret_cast<__nv_bfloat16*>(w_bf16), adam_m, adam_v, lr, beta1, beta2, eps, bc1, bc2,
-      1);
-  return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
+  const cudaError_t e = launch_reduce(scratch, scratch + (size_t)nblk * NP, nblk, batch, nullptr,
+                                      loss, master, w_bf16, adam_m, adam_v, lr, beta1, beta2, eps,
+                                      bc1, bc2, 1, (cudaStream_t)stream);
+  return e == cudaSuccess ? PIC_OK : PIC_ECUDA;
 }
 
 }  // extern "C"
