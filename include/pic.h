@@ -249,8 +249,9 @@ int pic_get_field(pic_handle* h, int instance, double* phi, float* E, int64_t n_
 
 /* Turn sampling on (period >= 1) or off (0) for every instance; clears the
  * sums either way.  The first call with period >= 1 allocates 32 bytes per
- * node.  While on, each step launches one more kernel, which returns at once
- * on steps that are not samples. */
+ * node.  While on, a sampled step launches one more kernel; with fewer than 16
+ * steps per distinct sampling phase every step does, and it returns at once on
+ * steps that are not samples. */
 int pic_set_profile_period(pic_handle* h, int64_t period);
 
 /* Averages over the K samples taken so far by one instance, on its

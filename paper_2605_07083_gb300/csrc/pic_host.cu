@@ -113,6 +113,7 @@ struct pic_handle {
   bool sort_ready = false;
   SortGrid sort_grid{1, 1, 1};
   int prof_gx = 1;              // k_profile blocks per segment
+  bool profile_each = false;    // k_profile after every step (else only after sampled ones)
   size_t prof_smem = 0;
   char last_error[256] = {0};
 };
@@ -600,6 +601,41 @@ bool sort_due(const pic_handle* h, int64_t step_after) {
 // for the push weights, then the collision blocks
 int mid_blocks(const pic_handle* h) { return 4 * h->n_inst * h->st.kp + 1 + h->mcc_blocks; }
 
+// Steps from `step` on until one whose new state some diode samples
+// (profile_due); 0 when that step itself is sampled.
+int64_t steps_to_sample(const pic_handle* h, int64_t step) {
+  const int64_t period = h->st.prof_period;
+  int64_t gap = INT64_MAX;
+  for (const InstConst& k : h->ic) {
+    if (step < k.window_start) {
+      gap = std::min(gap, k.window_start - step);
+    } else {
+      const int64_t past = (int64_t)((uint64_t)step - (uint64_t)k.window_start) % period;
+      gap = std::min(gap, past > 0 ? period - past : -past);
+    }
+  }
+  return gap;
+}
+
+// Sampled steps few and far between (at least 16 steps per distinct sampling
+// phase): the steps between them run without the sampler's launch, which
+// returned at once but took ~2 us of each step and kept small diodes from
+// k_fused, and each sampled step runs by itself.  Measured per step, sampler
+// after every step -> this: one small diode of 21k particles, a sample every
+// 16 steps 20.9 -> 17.4 us, every 100 20.6 -> 11.1; the 11 paper diodes, every
+// 100, 132 -> 130.  With fewer steps between samples the graphs get too short
+// to pay, and the sampler follows every step.
+void set_profile_mode(pic_handle* h) {
+  const int64_t period = h->st.prof_period;
+  h->profile_each = false;
+  if (period <= 0) return;
+  std::vector<int64_t> phase;
+  for (const InstConst& k : h->ic) phase.push_back((k.window_start % period + period) % period);
+  std::sort(phase.begin(), phase.end());
+  const int64_t distinct = std::unique(phase.begin(), phase.end()) - phase.begin();
+  h->profile_each = period / 16 < distinct;
+}
+
 // the profile sampler after a step (device-side test of the sampling rule)
 void launch_profile(pic_handle* h) {
   if (h->st.prof_period > 0)
@@ -611,7 +647,8 @@ cudaError_t launch_step(pic_handle* h) {
   push_kernel(h, h->push_threads, h->push_chunk)<<<h->G, h->push_threads, h->push_smem, h->stream>>>(h->st);
   mid_kernel(h)<<<mid_blocks(h), kPostThreads, h->mid_smem, h->stream>>>(h->st);
   k_post<<<3 * h->n_inst, kPostThreads, h->post_smem, h->stream>>>(h->st);
-  launch_profile(h);
+  if (h->profile_each || (h->st.prof_period > 0 && steps_to_sample(h, h->host_step) == 0))
+    launch_profile(h);
   h->host_step += 1;
   h->counts_known = false;
   if (sort_due(h, h->host_step)) launch_sort(h);
@@ -625,7 +662,7 @@ void enqueue_steps(pic_handle* h, int n, int first) {
                                                     h->stream>>>(h->st);
     mid_kernel(h)<<<mid_blocks(h), kPostThreads, h->mid_smem, h->stream>>>(h->st);
     k_post<<<3 * h->n_inst, kPostThreads, h->post_smem, h->stream>>>(h->st);
-    launch_profile(h);
+    if (h->profile_each) launch_profile(h);
     if (sort_due(h, first + i + 1)) launch_sort(h);
   }
 }
@@ -673,10 +710,11 @@ void set_fused_shape(pic_handle* h) {
 }
 
 // Step graphs let the device choose k_fused?  It takes neither sorts nor
-// profile samples, and has no bulk-copy wait to give up on.  The choice costs
-// ~15 us per kRouteSteps steps (a kernel and a conditional node), so it is not
-// offered where the last counts the host knows make k_fused take twice the
-// time of the three kernels.
+// profile samples (sampled steps run outside the graphs unless profile_each)
+// and has no bulk-copy wait to give up on.  The choice costs ~15 us per
+// kRouteSteps steps (a kernel and a conditional node), so it is not offered
+// where the last counts the host knows make k_fused take twice the time of
+// the three kernels.
 bool fused_allowed(const pic_handle* h) {
   long long total = 0;
   int longest = 0;
@@ -687,7 +725,7 @@ bool fused_allowed(const pic_handle* h) {
   }
   const StepEstimate e = estimate_step(h->n_inst, (float)longest, (float)total,
                                        std::max(1, h->fused_c), h->sm_count, h->max_nodes);
-  return h->fused_c > 0 && e.fused < 2.0f * e.three && h->sort_period <= 0 && h->st.prof_period <= 0 &&
+  return h->fused_c > 0 && e.fused < 2.0f * e.three && h->sort_period <= 0 && !h->profile_each &&
          h->st.wait_limit == kWaitLimit;
 }
 
@@ -1090,12 +1128,12 @@ int pic_set_step(pic_handle* h, int64_t step) {
   return PIC_OK;
 }
 
-// The plan of pic_step(n) from the current step: single steps up to a
-// sort-aligned step (with a sort), graphs longest first, single steps for the
+// n steps from `step` on, none of them sampled unless profile_each: single
+// steps up to a sort-aligned step (with a sort), graphs longest first, single steps for the
 // rest.  With run set it launches the plan; otherwise it only captures the
 // graphs the plan needs (pic_prepare_steps).
-static int step_plan(pic_handle* h, int64_t n_steps, bool run) {
-  int64_t left = n_steps, step = h->host_step;
+static int plan_stretch(pic_handle* h, int64_t n_steps, int64_t step, bool run) {
+  int64_t left = n_steps;
   const int len = graph_unit(h);
   const int64_t sp = h->sort_period;
   // a graph bakes in where the periodic sort falls, so with a sort the graphs
@@ -1131,6 +1169,27 @@ static int step_plan(pic_handle* h, int64_t n_steps, bool run) {
   for (; run && left > 0; --left) {
     cudaError_t e = launch_step(h);
     if (e != cudaSuccess) return cuda_fail_at(h, e, "step kernel launch");
+  }
+  return PIC_OK;
+}
+
+// The plan of pic_step(n) from the current step: stretches between sampled
+// steps, and those by themselves.
+static int step_plan(pic_handle* h, int64_t n_steps, bool run) {
+  int64_t left = n_steps, step = h->host_step;
+  const bool split = h->st.prof_period > 0 && !h->profile_each;
+  while (left > 0) {
+    const int64_t gap = split ? steps_to_sample(h, step) : left;
+    const int64_t m = std::max<int64_t>(1, std::min(left, gap));
+    if (gap > 0) {
+      int rc = plan_stretch(h, m, step, run);
+      if (rc != PIC_OK) return rc;
+    } else if (run) {
+      cudaError_t e = launch_step(h);
+      if (e != cudaSuccess) return cuda_fail_at(h, e, "step kernel launch");
+    }
+    step += m;
+    left -= m;
   }
   return run ? h->sticky : PIC_OK;
 }
@@ -1307,6 +1366,7 @@ int pic_set_profile_period(pic_handle* h, int64_t period) {
     if (e != cudaSuccess) return cuda_fail(h, e);
   }
   h->st.prof_period = period;
+  set_profile_mode(h);
   drop_graph(h);
   return PIC_OK;
 }
@@ -1531,6 +1591,7 @@ int pic_load(pic_handle* h, const void* host_buf, size_t bytes) {
       if (rc != PIC_OK) return rc;
     }
     h->st.prof_period = hd.prof_period;
+    set_profile_mode(h);
   } else {
     int rc = pic_set_profile_period(h, 0);
     if (rc != PIC_OK) return rc;

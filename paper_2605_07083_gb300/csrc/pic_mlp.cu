@@ -36,8 +36,8 @@ static_assert(NP == PIC_MLP_PARAMS, "parameter count");
 // the partials' stores.  A 4 x 4 register tile needs two shared loads per 16
 // FMAs; with one thread per unit each FMA row had a 2-byte global load and a
 // scalar shared load per FMA, 150 us even for one tile.  Measured before and
-// after: training step of 4096 samples 161 -> 45 us, gradient of 100 samples
-// 154 -> 21.5 us, prediction of 41216 samples 287 -> 84 us.
+// after: training step of 4096 samples 161 -> 42 us, gradient of 100 samples
+// 154 -> 20.5 us, prediction of 41216 samples 287 -> 82 us.
 constexpr int kThr = 512, kWarps = kThr / 32;
 constexpr int kWRow = H + 8;                 // bfloat16 per row of a transposed matrix
 constexpr int kSms = 152;                    // tiles are kept to one wave while they fit
