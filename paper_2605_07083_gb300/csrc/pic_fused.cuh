@@ -151,7 +151,7 @@ __device__ __forceinline__ int fused_push(const DevState& st, FusedShared& S, co
       zp[q] = z4;
       vp[q] = v4;
       if (dm == 0u) {
-        deposit_quad(hist, z4, c.inv_dz, c.Nz);
+        deposit_quad(hist, z4, c.inv_dz, c.Nz, false);
       } else {
         const float z[4] = {z4.x, z4.y, z4.z, z4.w};
 #pragma unroll
