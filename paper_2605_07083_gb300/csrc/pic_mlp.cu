@@ -686,7 +686,7 @@ constexpr int kRedThreads = 128, kRedUnroll = 16;   // 16 partials in flight per
 
 // grad[p] = sum over CTAs of the partials (fixed order); optional Adam update
 // of the FP32 master with the bfloat16 copy re-rounded (Kingma & Ba 2015).
-__global__ void k_mlp_reduce_adam(const float* __restrict__ part, const float* __restrict__ lpart,
+__global__ void k_mlp_reduce_adam(const float* part, const float* lpart,
                                   int n_part, long long batch, float* __restrict__ grad,
                                   float* __restrict__ loss, float* __restrict__ master,
                                   __nv_bfloat16* __restrict__ w, float* __restrict__ m,
@@ -694,7 +694,8 @@ __global__ void k_mlp_reduce_adam(const float* __restrict__ part, const float* _
                                   float eps, float bc1, float bc2, int do_adam) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   // launched while the tiles still run (launch_reduce): everything below reads
-  // what they, or launches before them, wrote
+  // what they, or launches before them, wrote (the partials through plain
+  // loads: they change during this kernel's life, so no __restrict__ const)
   cudaGridDependencySynchronize();
   if (p == 0 && loss) {
     float L = 0.0f;
