@@ -6,8 +6,8 @@
 // blocks, by how many diodes share the chip) owns a diode and runs n_steps of
 // it: field, constants, counts and tallies stay in shared memory, the
 // particles in L2, and the phases of a step meet at hardware cluster
-// barriers (10.4 us a step; 128 diodes of 5.5k particles 32.4 -> 11.7 us).  What is left
-// is the phases' own round trips: about 40 % push, the rest lists, charge,
+// barriers (9.4 us a step; 128 diodes of 5.5k particles 32.4 -> 11.4 us).  What
+// is left is the phases' own round trips: about 40 % push, the rest lists, charge,
 // field and compaction, of which only latency counts; a block keeps its
 // registers below the limit, since a spilled one is fetched from L2 after
 // every barrier (768 threads, which spill, took 28 us).  It computes exactly
@@ -47,11 +47,12 @@ constexpr int kFusedTeamWarps = kFusedWarps - 1;   // warps of phase D's teams
 
 // shared memory: (E_j, dE_j) pairs, E, two histograms, the blocks' and the
 // diode's node charge (up to kFusedWarpCells cells every block writes its own
-// into all of them, else they are read from it), the candidate list, the absorbed lists (three species;
-// a warp's share of them), the event keys of two species
+// into all of them, else they are read from it), the candidate list, the absorbed
+// lists (three species; a warp's share of them), the event keys of two species
 __host__ __device__ constexpr size_t fused_smem(int nodes) {
   return (size_t)((nodes + 3) & ~3) *
-             (8 + 4 + 12 + 12 + 16 + 8 * (nodes <= kFusedWarpCells + 1 ? kFusedMaxC : 1)) + (size_t)kFusedCand * 16 +
+             (8 + 4 + 12 + 12 + 16 + 8 * (nodes <= kFusedWarpCells + 1 ? kFusedMaxC : 1)) +
+         (size_t)kFusedCand * 16 +
          (size_t)3 * kFusedList * 4 + (size_t)3 * kFusedWarps * kFusedWarpList * 4 +
          (size_t)2 * kEvCap * 8;
 }
