@@ -1581,10 +1581,9 @@ int pic_load(pic_handle* h, const void* host_buf, size_t bytes) {
   for (const InstDyn& d : dyn)
     if (d.step != hd.step) return PIC_EINVAL;
   if (ckpt_bytes(h, counts, hd.has_prof != 0) > bytes) return PIC_EINVAL;
-  // validated: from here on the handle takes the checkpoint's state
-  h->counts_known = true;
-  h->known_count = counts;
-  for (int i = 0; i < h->n_inst; ++i) h->known_id[i] = dyn[i].next_id;
+  // validated: from here on the handle takes the checkpoint's state.  What
+  // follows can fail, so the counts are the device's own until it is all there.
+  h->counts_known = false;
   if (hd.has_prof) {
     if (!h->st.phi_sum) {          // allocate the sums (overwritten below)
       int rc = pic_set_profile_period(h, 1);
@@ -1620,6 +1619,9 @@ int pic_load(pic_handle* h, const void* host_buf, size_t bytes) {
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e);
+  h->counts_known = true;
+  h->known_count = counts;
+  for (int i = 0; i < h->n_inst; ++i) h->known_id[i] = dyn[i].next_id;
   h->host_step = hd.step;
   h->dirty = true;               // charge and field are recomputed from the particles
   drop_graph(h);
