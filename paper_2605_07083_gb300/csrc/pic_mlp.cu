@@ -684,8 +684,12 @@ __global__ void __launch_bounds__(kThr, 1) k_mlp_fwd_bwd(const float* __restrict
 
 constexpr int kRedThreads = 128, kRedUnroll = 16;   // 16 partials in flight per thread
 
-// grad[p] = sum over CTAs of the partials (fixed order); optional Adam update
-// of the FP32 master with the bfloat16 copy re-rounded (Kingma & Ba 2015).
+// grad[p] = sum over CTAs of the partials; optional Adam update of the FP32
+// master with the bfloat16 copy re-rounded (Kingma & Ba 2015).  The order is
+// fixed: sixteen sums of every sixteenth partial, then their tree.  (The tiles
+// of 8 or 16 samples that a batch of less than a wave is cut into are up to
+// four times as many partials as tiles of 32; one after another, 152 of them
+// have an error of up to 150 roundings of the sum, so 13 here.)
 __global__ void k_mlp_reduce_adam(const float* part, const float* lpart,
                                   int n_part, long long batch, float* __restrict__ grad,
                                   float* __restrict__ loss, float* __restrict__ master,
@@ -697,22 +701,32 @@ __global__ void k_mlp_reduce_adam(const float* part, const float* lpart,
   // what they, or launches before them, wrote (the partials through plain
   // loads: they change during this kernel's life, so no __restrict__ const)
   cudaGridDependencySynchronize();
-  if (p == 0 && loss) {
+  if (p < 32 && loss) {                        // the first warp, whole
     float L = 0.0f;
-    for (int b = 0; b < n_part; ++b) L += lpart[b];
-    *loss = L / (float)(batch * OUT);
+    for (int b = p; b < n_part; b += 32) L += lpart[b];
+    for (int off = 16; off > 0; off >>= 1) L += __shfl_down_sync(0xffffffffu, L, off);
+    if (p == 0) *loss = L / (float)(batch * OUT);
   }
   if (p >= NP) return;
-  float gsum = 0.0f;
+  float sum[kRedUnroll];
+#pragma unroll
+  for (int u = 0; u < kRedUnroll; ++u) sum[u] = 0.0f;
   int b = 0;
   for (; b + kRedUnroll <= n_part; b += kRedUnroll) {
-    float v[kRedUnroll];
+    float x[kRedUnroll];
 #pragma unroll
-    for (int u = 0; u < kRedUnroll; ++u) v[u] = part[(size_t)(b + u) * NP + p];
+    for (int u = 0; u < kRedUnroll; ++u) x[u] = part[(size_t)(b + u) * NP + p];
 #pragma unroll
-    for (int u = 0; u < kRedUnroll; ++u) gsum += v[u];
+    for (int u = 0; u < kRedUnroll; ++u) sum[u] += x[u];
   }
-  for (; b < n_part; ++b) gsum += part[(size_t)b * NP + p];
+#pragma unroll
+  for (int u = 0; u < kRedUnroll - 1; ++u)
+    if (b + u < n_part) sum[u] += part[(size_t)(b + u) * NP + p];
+#pragma unroll
+  for (int w = kRedUnroll / 2; w > 0; w >>= 1)
+#pragma unroll
+    for (int u = 0; u < w; ++u) sum[u] += sum[u + w];
+  const float gsum = sum[0];
   if (grad) grad[p] = gsum;
   if (!do_adam) return;
   const float mm = beta1 * m[p] + (1.0f - beta1) * gsum;
