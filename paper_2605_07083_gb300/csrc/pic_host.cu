@@ -737,7 +737,7 @@ int add_routed_steps(pic_handle* h, cudaGraph_t g, int n, cudaGraphNode_t* tail)
   cudaGraphConditionalHandle cond;
   cudaError_t e = cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault);
   if (e != cudaSuccess) return cuda_fail_at(h, e, "cudaGraphConditionalHandleCreate");
-  // most a diode can gain: its emission, and two particles per ionisation event
+  // most a diode can gain by emission and ionisation (two particles an event)
   long long growth = 0;
   for (const InstConst& k : h->ic)
     growth = std::max(growth, (long long)n * (k.emit_floor + 1 + 2 * kEvCap));
