@@ -312,10 +312,11 @@ void note_counts(pic_handle* h, int instance) {
   for (int s = 0; s < 3; ++s) h->known_count[3 * instance + s] = h->rb->count[s];
 }
 
-// Device arrays that a kernel may read or write: device or managed memory,
-// aligned to their elements.  Anything else goes through cudaMemcpyAsync,
-// which handles it or refuses it.  *vec: all are 16-byte aligned.
-bool kernel_arrays(std::initializer_list<const void*> ps, bool* vec) {
+// Device arrays that a kernel on `device` may read or write: that device's own
+// or managed memory, aligned to their elements.  Anything else (another
+// device's memory without peer access, say) goes through cudaMemcpyAsync, which
+// handles it or refuses it.  *vec: all are 16-byte aligned.
+bool kernel_arrays(std::initializer_list<const void*> ps, int device, bool* vec) {
   *vec = true;
   for (const void* p : ps) {
     if (!p) continue;
@@ -326,7 +327,8 @@ bool kernel_arrays(std::initializer_list<const void*> ps, bool* vec) {
       cudaGetLastError();
       return false;
     }
-    if (a.type != cudaMemoryTypeDevice && a.type != cudaMemoryTypeManaged) return false;
+    if (a.type != cudaMemoryTypeManaged && (a.type != cudaMemoryTypeDevice || a.device != device))
+      return false;
   }
   return true;
 }
@@ -1085,7 +1087,7 @@ int pic_inject(pic_handle* h, int instance, int species, int64_t n, const float*
   // lies in [0, L), so a rejected call leaves the instance as it was
   const int64_t base = h->seg_off[g] + count;
   bool vec = true;
-  const bool direct = on_device && kernel_arrays({z, vx, vy, vz}, &vec);
+  const bool direct = on_device && kernel_arrays({z, vx, vy, vz}, h->device, &vec);
   if (!direct) {
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const size_t bytes = sizeof(float) * (size_t)n;
@@ -1287,7 +1289,7 @@ int pic_get_state(pic_handle* h, int instance, int species, float* z, float* vx,
     return PIC_EINVAL;
   const int g = 3 * instance + species;
   bool vec = false;
-  if (on_device && kernel_arrays({z, vx, vy, vz, id}, &vec)) {
+  if (on_device && kernel_arrays({z, vx, vy, vz, id}, h->device, &vec)) {
     const int64_t room = std::max<int64_t>(1, std::min<int64_t>(cap, h->seg_cap[g]));
     const unsigned blocks =
         (unsigned)std::min<int64_t>((room + 1023) / 1024, (int64_t)8 * h->sm_count);

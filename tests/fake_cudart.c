@@ -1,0 +1,130 @@
+/* A stand-in for the CUDA runtime with two devices and no GPU, for the host
+ * side of the library: memory is the host's, launches run nothing.  It keeps
+ * what the tests look at -- the current device, launches on a stream of
+ * another device (refused, as the runtime does), copies, the device on which
+ * each kernel attribute was set -- and answers pointer queries from a table
+ * that the test fills in. */
+#include <stddef.h>
+#include <stdint.h>
+#include <stdlib.h>
+#include <string.h>
+
+typedef struct { unsigned x, y, z; } dim3;
+typedef struct { int type, device; void* device_pointer; void* host_pointer; long reserved[8]; } Attributes;
+
+enum { kInvalidValue = 1, kInvalidResourceHandle = 400, kStreamDevice1 = 0x1000 };
+
+int fake_device = 0;          /* the current device of the only thread */
+int fake_launches = 0, fake_copies = 0, fake_refused = 0;
+int fake_attributes[2] = {0, 0};
+static int last_error = 0;
+static struct { const char* p; size_t bytes; int type, device; } table[16];
+static int entries = 0;
+
+void fake_array(const void* p, size_t bytes, int type, int device) {
+  table[entries].p = p;
+  table[entries].bytes = bytes;
+  table[entries].type = type;
+  table[entries++].device = device;
+}
+
+int cudaGetDevice(int* d) { *d = fake_device; return 0; }
+int cudaSetDevice(int d) { if (d < 0 || d > 1) return 101; fake_device = d; return 0; }
+int cudaDeviceGetAttribute(int* v, int attr, int device) {
+  (void)device;
+  *v = attr == 16 ? 152 : attr == 97 ? 232448 : 0;   /* multiprocessors, opt-in shared memory */
+  return 0;
+}
+int cudaGetLastError(void) { int e = last_error; last_error = 0; return e; }
+const char* cudaGetErrorString(int e) { (void)e; return "fake"; }
+
+int cudaPointerGetAttributes(Attributes* a, const void* p) {
+  memset(a, 0, sizeof *a);
+  for (int i = 0; i < entries; ++i)
+    if ((const char*)p >= table[i].p && (const char*)p < table[i].p + table[i].bytes) {
+      a->type = table[i].type;
+      a->device = table[i].device;
+    }
+  return 0;
+}
+
+int cudaMallocAsync(void** p, size_t n, void* s) { (void)s; *p = aligned_alloc(256, (n + 255) & ~(size_t)255); return 0; }
+int cudaFreeAsync(void* p, void* s) { (void)s; free(p); return 0; }
+int cudaHostAlloc(void** p, size_t n, unsigned f) { (void)f; *p = calloc(1, n); return 0; }
+int cudaFreeHost(void* p) { free(p); return 0; }
+int cudaMemcpyAsync(void* d, const void* s, size_t n, int kind, void* st) {
+  (void)kind; (void)st;
+  memmove(d, s, n);
+  ++fake_copies;
+  return 0;
+}
+int cudaMemsetAsync(void* d, int v, size_t n, void* s) { (void)s; memset(d, v, n); return 0; }
+int cudaStreamCreateWithFlags(void** s, unsigned f) { (void)f; *s = (void*)0x2000; return 0; }
+int cudaStreamDestroy(void* s) { (void)s; return 0; }
+int cudaStreamSynchronize(void* s) { (void)s; return 0; }
+
+int cudaFuncGetAttributes(void* a, const void* f) { (void)f; memset(a, 0, 4 * sizeof(size_t)); return 0; }
+int cudaFuncSetAttribute(const void* f, int attr, int v) {
+  (void)f; (void)attr; (void)v;
+  ++fake_attributes[fake_device];
+  return 0;
+}
+int cudaGetSymbolAddress(void** p, const void* s) { (void)s; static int word[4]; *p = word; return 0; }
+int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* f, int t, size_t m, unsigned fl) {
+  (void)f; (void)t; (void)m; (void)fl;
+  *n = 2;
+  return 0;
+}
+int cudaOccupancyMaxActiveClusters(int* n, const void* f, const void* cfg) { (void)f; (void)cfg; *n = 8; return 0; }
+
+static int launch(void* stream) {
+  if (stream == (void*)kStreamDevice1 && fake_device != 1) {
+    ++fake_refused;
+    return last_error = kInvalidResourceHandle;
+  }
+  ++fake_launches;
+  return 0;
+}
+static void* pushed_stream;
+unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t m, void* s) {
+  (void)g; (void)b; (void)m;
+  pushed_stream = s;
+  return 0;
+}
+int __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* m, void** s) {
+  g->x = g->y = g->z = b->x = b->y = b->z = 1;
+  *m = 0;
+  *s = pushed_stream;
+  return 0;
+}
+int __cudaGetKernel(void** k, const void* f) { *k = (void*)f; return 0; }
+int __cudaLaunchKernel(void* k, dim3 g, dim3 b, void** a, size_t m, void* s) {
+  (void)k; (void)g; (void)b; (void)a; (void)m;
+  return launch(s);
+}
+typedef struct { dim3 grid, block; size_t smem; void* stream; void* attrs; unsigned n; } Config;
+int cudaLaunchKernelExC(const Config* c, const void* f, void** a) { (void)f; (void)a; return launch(c->stream); }
+
+void** __cudaRegisterFatBinary(void* p) { (void)p; static void* h; return &h; }
+void __cudaRegisterFatBinaryEnd(void** h) { (void)h; }
+void __cudaUnregisterFatBinary(void** h) { (void)h; }
+void __cudaRegisterFunction(void) {}
+void __cudaRegisterVar(void) {}
+
+/* not reached by these tests */
+int cudaEventCreate(void** e) { *e = NULL; return kInvalidValue; }
+int cudaEventDestroy(void* e) { (void)e; return 0; }
+int cudaEventElapsedTime(float* t, void* a, void* b) { (void)a; (void)b; *t = 0; return kInvalidValue; }
+int cudaEventRecord(void* e, void* s) { (void)e; (void)s; return kInvalidValue; }
+int cudaEventSynchronize(void* e) { (void)e; return kInvalidValue; }
+int cudaGraphAddKernelNode(void) { return kInvalidValue; }
+int cudaGraphAddNode(void) { return kInvalidValue; }
+int cudaGraphConditionalHandleCreate(void) { return kInvalidValue; }
+int cudaGraphCreate(void) { return kInvalidValue; }
+int cudaGraphDestroy(void) { return 0; }
+int cudaGraphExecDestroy(void) { return 0; }
+int cudaGraphInstantiate(void) { return kInvalidValue; }
+int cudaGraphLaunch(void) { return kInvalidValue; }
+int cudaStreamBeginCapture(void) { return kInvalidValue; }
+int cudaStreamBeginCaptureToGraph(void) { return kInvalidValue; }
+int cudaStreamEndCapture(void) { return kInvalidValue; }

@@ -1,0 +1,69 @@
+"""What the library's host side does in a process with two devices, on a
+stand-in for the CUDA runtime (fake_cudart.c): no GPU, nothing is launched.
+Each case runs in a process of its own, which loads the library against the
+stand-in."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+from conftest import ROOT
+
+DEVICE, MANAGED = 2, 3                       # cudaMemoryType
+HANDLE = '''
+import ctypes as C, sys
+lib = C.CDLL(sys.argv[1])
+fake = C.CDLL("libcudart.so.13")
+word = lambda name: C.c_int.in_dll(fake, name)
+from paper_2605_07083_gb300 import pic, workloads as W
+for name, (res, args) in pic.ENTRY_POINTS.items():
+    getattr(lib, name).restype, getattr(lib, name).argtypes = res, args
+fake.fake_array.argtypes = [C.c_void_p, C.c_size_t, C.c_int, C.c_int]
+def create():                                # on device 1, with a stream of device 1
+    word("fake_device").value = 1
+    h, cfg = C.c_void_p(), pic.make_config(dict(W.single_diode_small(), capacity=(4096,) * 3))
+    assert lib.pic_create(C.byref(cfg), 1, C.c_void_p(0x1000), None, C.byref(h)) == 0
+    return h
+def array(n, kind, device):
+    a = (C.c_uint32 * n)()
+    fake.fake_array(a, C.sizeof(a), kind, device)
+    return a
+'''
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    from paper_2605_07083_gb300 import build as B
+    lib = B.build()
+    out = tmp_path_factory.mktemp("fake")
+    subprocess.run(["gcc", "-O1", "-shared", "-fPIC", "-Wno-builtin-declaration-mismatch",
+                    "-Wl,-soname,libcudart.so.13", os.path.join(ROOT, "tests", "fake_cudart.c"),
+                    "-o", str(out / "libcudart.so.13")], check=True)
+
+    def go(body):
+        env = dict(os.environ, LD_LIBRARY_PATH=str(out), PYTHONPATH=ROOT)
+        r = subprocess.run([sys.executable, "-c", HANDLE + body, lib], env=env, text=True,
+                           capture_output=True, timeout=120)
+        assert r.returncode == 0, r.stdout + r.stderr
+    return go
+
+
+@pytest.mark.parametrize("kind,device,direct", [(DEVICE, 1, True), (DEVICE, 0, False),
+                                                (MANAGED, 0, True), (0, 0, False)])
+def test_only_arrays_of_the_handles_device_are_read_by_kernels(run, kind, device, direct):
+    """One array of several elsewhere (or not known to the runtime) sends the
+    whole call through cudaMemcpyAsync, which carries it over or refuses it."""
+    run(f'''
+h = create()
+a = [array(512, {DEVICE}, 1) for _ in range(4)] + [array(512, {kind}, {device})]
+n = C.c_int64()
+copies = word("fake_copies").value
+assert lib.pic_inject(h, 0, 0, 512, a[0], a[1], a[4], a[3], 1) == 0
+assert (word("fake_copies").value == copies) == {direct}
+# the counts come from kernels, which the stand-in does not run: no particles
+# to copy, and one launch either way
+launches = word("fake_launches").value
+assert lib.pic_get_state(h, 0, 0, *a, 512, C.byref(n), 1) == 0
+assert word("fake_launches").value == launches + 1
+''')
