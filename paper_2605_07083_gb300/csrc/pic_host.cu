@@ -283,6 +283,22 @@ void readback_give(Readback* r) {
   cudaFreeHost(r);
 }
 
+// The handle's device is current while this lives: a launch on a stream of
+// another device is refused, and the calls that only read may come from a
+// thread that has never selected one (cudaMemcpyAsync, with which they read
+// once, takes any).
+struct OnDevice {
+  int before = -1;
+  explicit OnDevice(const pic_handle* h) {
+    int now = 0;
+    if (cudaGetDevice(&now) == cudaSuccess && now != h->device && cudaSetDevice(h->device) == cudaSuccess)
+      before = now;
+  }
+  ~OnDevice() {
+    if (before >= 0) cudaSetDevice(before);
+  }
+};
+
 // wait for the readback kernel just launched
 int read_done(pic_handle* h) {
   cudaError_t e = cudaGetLastError();
@@ -302,6 +318,7 @@ int flags_of(pic_handle* h) {
 }
 
 int check_flags(pic_handle* h) {
+  OnDevice on(h);
   k_read<<<1, 256, 0, h->stream>>>(h->st, -1, h->rb);
   int rc = read_done(h);
   return rc == PIC_OK ? flags_of(h) : rc;
@@ -1275,6 +1292,7 @@ int pic_profile_steps(pic_handle* h, int64_t n_steps, pic_profile* out) {
 
 int pic_diagnostics(pic_handle* h, int instance, pic_diag* out) {
   if (!h || !out || instance < 0 || instance >= h->n_inst) return PIC_EINVAL;
+  OnDevice on(h);
   k_read<<<1, 256, 0, h->stream>>>(h->st, instance, h->rb);
   int rc = read_done(h);
   if (rc != PIC_OK) return rc;
@@ -1288,6 +1306,7 @@ int pic_get_state(pic_handle* h, int instance, int species, float* z, float* vx,
   if (!h || !n || instance < 0 || instance >= h->n_inst || species < 0 || species > 2)
     return PIC_EINVAL;
   const int g = 3 * instance + species;
+  OnDevice on(h);
   bool vec = false;
   if (on_device && kernel_arrays({z, vx, vy, vz, id}, h->device, &vec)) {
     const int64_t room = std::max<int64_t>(1, std::min<int64_t>(cap, h->seg_cap[g]));
@@ -1327,6 +1346,7 @@ int pic_get_rho_fixed(pic_handle* h, int instance, int64_t* out, int64_t n_nodes
   if (n_nodes < nn) return PIC_EINVAL;
   int rc = ensure_field(h);
   if (rc != PIC_OK) return rc;
+  OnDevice on(h);
   k_read_rho<<<1, 512, 0, h->stream>>>(h->st, instance, h->rb);
   rc = read_done(h);
   if (rc != PIC_OK) return rc;

@@ -67,3 +67,23 @@ launches = word("fake_launches").value
 assert lib.pic_get_state(h, 0, 0, *a, 512, C.byref(n), 1) == 0
 assert word("fake_launches").value == launches + 1
 ''')
+
+
+@pytest.mark.parametrize("call", [
+    "lib.pic_synchronize(h)", "lib.pic_diagnostics(h, 0, C.byref(pic.PicDiag()))",
+    "lib.pic_get_state(h, 0, 0, *a, 512, C.byref(n), 1)",
+    "lib.pic_get_state(h, 0, 0, None, None, None, None, None, 512, C.byref(n), 0)",
+    "lib.pic_get_rho_fixed(h, 0, rho, 129)", "lib.pic_checkpoint_bytes(h, C.byref(size))"])
+def test_reads_work_whichever_device_is_current(run, call):
+    """A thread that reads a handle need not have selected the handle's device
+    (launches on another device's stream are refused), and finds its own device
+    current afterwards."""
+    run(f'''
+h = create()
+a = [array(512, {DEVICE}, 1) for _ in range(5)]
+n, size, rho = C.c_int64(), C.c_size_t(), (C.c_int64 * 129)()
+assert lib.pic_get_rho_fixed(h, 0, rho, 129) == 0      # the empty state's charge is deposited
+word("fake_device").value = 0
+assert {call} == 0
+assert word("fake_refused").value == 0 and word("fake_device").value == 0
+''')
