@@ -786,16 +786,23 @@ constexpr size_t wide_smem(int warps) {
   return sizeof(WideSmem) + (size_t)warps * kWideBuf * sizeof(float);
 }
 
+// the kernels' shared-memory limits, once for every device (the attribute is
+// the current device's)
 bool prepare_kernels() {
-  static bool done = false;
-  if (!done)
-    done = forward_limit<8>() == cudaSuccess && forward_limit<16>() == cudaSuccess &&
-           forward_limit<32>() == cudaSuccess &&
-           cudaFuncSetAttribute(k_mlp_forward_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)wide_smem(kWideMaxWarps)) == cudaSuccess &&
-           grad_limit<8>() == cudaSuccess && grad_limit<16>() == cudaSuccess &&
-           grad_limit<32>() == cudaSuccess;
-  return done;
+  static bool done[64] = {false};
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess) return false;
+  const bool known = device >= 0 && device < 64;
+  if (known && done[device]) return true;
+  const bool ok = forward_limit<8>() == cudaSuccess && forward_limit<16>() == cudaSuccess &&
+                  forward_limit<32>() == cudaSuccess &&
+                  cudaFuncSetAttribute(k_mlp_forward_wide,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)wide_smem(kWideMaxWarps)) == cudaSuccess &&
+                  grad_limit<8>() == cudaSuccess && grad_limit<16>() == cudaSuccess &&
+                  grad_limit<32>() == cudaSuccess;
+  if (ok && known) done[device] = true;
+  return ok;
 }
 
 // The reduction's launch overlaps the end of the tiles (programmatic stream

@@ -87,3 +87,19 @@ word("fake_device").value = 0
 assert {call} == 0
 assert word("fake_refused").value == 0 and word("fake_device").value == 0
 ''')
+
+
+def test_network_kernels_are_set_up_on_every_device(run):
+    """The raised shared-memory limit of a kernel holds for one device: the
+    first call on a second one sets it there, later calls on neither."""
+    run(f'''
+a = array(1 << 16, {DEVICE}, 0)
+counts = (C.c_int * 2).in_dll(fake, "fake_attributes")
+for device in (0, 1, 1, 0):
+    word("fake_device").value = device
+    assert lib.pic_mlp_forward(a, a, a, 10, a, None) == 0
+    seen = list(counts)
+    if device == 1:
+        assert seen[1] == seen[0] > 0
+assert list(counts) == seen
+''')
