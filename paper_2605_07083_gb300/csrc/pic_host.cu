@@ -329,23 +329,53 @@ void note_counts(pic_handle* h, int instance) {
   for (int s = 0; s < 3; ++s) h->known_count[3 * instance + s] = h->rb->count[s];
 }
 
-// Device arrays that a kernel on `device` may read or write: that device's own
-// or managed memory, aligned to their elements.  Anything else (another
-// device's memory without peer access, say) goes through cudaMemcpyAsync, which
-// handles it or refuses it.  *vec: all are 16-byte aligned.
-bool kernel_arrays(std::initializer_list<const void*> ps, int device, bool* vec) {
+// First and last byte + 1 of the allocation that p lies in (false: not known).
+bool allocation_of(const void* p, uintptr_t* lo, uintptr_t* hi) {
+  using Fn = int (*)(unsigned long long* base, size_t* bytes, unsigned long long p);
+  static const Fn fn = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault,
+                                         &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return (Fn)f;
+  }();
+  unsigned long long base = 0;
+  size_t bytes = 0;
+  if (!fn || fn(&base, &bytes, (unsigned long long)(uintptr_t)p) != 0) return false;
+  *lo = (uintptr_t)base;
+  *hi = (uintptr_t)base + bytes;
+  return true;
+}
+
+// Device arrays of `bytes` bytes that a kernel on `device` may read or write:
+// that device's own or managed memory, aligned to their elements, inside one
+// allocation.  Anything else (another device's memory without peer access, a
+// count that the array does not have) goes through cudaMemcpyAsync, which
+// handles it or refuses it where a kernel would fault.  *vec: all are 16-byte
+// aligned.
+bool kernel_arrays(std::initializer_list<const void*> ps, size_t bytes, int device, bool* vec) {
   *vec = true;
+  uintptr_t lo = 0, hi = 0;            // the allocation looked up last
   for (const void* p : ps) {
     if (!p) continue;
-    if ((uintptr_t)p & 3u) return false;
-    if ((uintptr_t)p & 15u) *vec = false;
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
+    const uintptr_t at = (uintptr_t)p;
+    if (at & 3u) return false;
+    if (at & 15u) *vec = false;
+    if (at < lo || at >= hi) {
+      cudaPointerAttributes a;
+      if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+      }
+      if (a.type != cudaMemoryTypeManaged && (a.type != cudaMemoryTypeDevice || a.device != device))
+        return false;
+      if (!allocation_of(p, &lo, &hi)) return false;
     }
-    if (a.type != cudaMemoryTypeManaged && (a.type != cudaMemoryTypeDevice || a.device != device))
-      return false;
+    if (bytes > hi - at) return false;
   }
   return true;
 }
@@ -1104,7 +1134,7 @@ int pic_inject(pic_handle* h, int instance, int species, int64_t n, const float*
   // lies in [0, L), so a rejected call leaves the instance as it was
   const int64_t base = h->seg_off[g] + count;
   bool vec = true;
-  const bool direct = on_device && kernel_arrays({z, vx, vy, vz}, h->device, &vec);
+  const bool direct = on_device && kernel_arrays({z, vx, vy, vz}, sizeof(float) * (size_t)n, h->device, &vec);
   if (!direct) {
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const size_t bytes = sizeof(float) * (size_t)n;
@@ -1308,8 +1338,9 @@ int pic_get_state(pic_handle* h, int instance, int species, float* z, float* vx,
   const int g = 3 * instance + species;
   OnDevice on(h);
   bool vec = false;
-  if (on_device && kernel_arrays({z, vx, vy, vz, id}, h->device, &vec)) {
-    const int64_t room = std::max<int64_t>(1, std::min<int64_t>(cap, h->seg_cap[g]));
+  const int64_t room = std::max<int64_t>(1, std::min<int64_t>(cap, h->seg_cap[g]));
+  if (on_device &&
+      kernel_arrays({z, vx, vy, vz, id}, sizeof(float) * (size_t)room, h->device, &vec)) {
     const unsigned blocks =
         (unsigned)std::min<int64_t>((room + 1023) / 1024, (int64_t)8 * h->sm_count);
     k_state_copy<<<blocks, 256, 0, h->stream>>>(h->st, g, cap, z, vx, vy, vz, id, vec ? 1 : 0, h->rb);

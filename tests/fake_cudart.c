@@ -48,6 +48,22 @@ int cudaPointerGetAttributes(Attributes* a, const void* p) {
   return 0;
 }
 
+static int address_range(unsigned long long* base, size_t* bytes, unsigned long long p) {
+  for (int i = 0; i < entries; ++i)
+    if ((const char*)(uintptr_t)p >= table[i].p && (const char*)(uintptr_t)p < table[i].p + table[i].bytes) {
+      *base = (unsigned long long)(uintptr_t)table[i].p;
+      *bytes = table[i].bytes;
+      return 0;
+    }
+  return kInvalidValue;
+}
+int cudaGetDriverEntryPointByVersion(const char* name, void** fn, unsigned version, unsigned long long flags, int* found) {
+  (void)version; (void)flags;
+  *fn = strcmp(name, "cuMemGetAddressRange") == 0 ? (void*)address_range : NULL;
+  *found = *fn ? 0 : 1;
+  return 0;
+}
+
 int cudaMallocAsync(void** p, size_t n, void* s) { (void)s; *p = aligned_alloc(256, (n + 255) & ~(size_t)255); return 0; }
 int cudaFreeAsync(void* p, void* s) { (void)s; free(p); return 0; }
 int cudaHostAlloc(void** p, size_t n, unsigned f) { (void)f; *p = calloc(1, n); return 0; }
@@ -77,12 +93,18 @@ int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* f
 }
 int cudaOccupancyMaxActiveClusters(int* n, const void* f, const void* cfg) { (void)f; (void)cfg; *n = 8; return 0; }
 
-static int launch(void* stream) {
+static struct { const void* f; const char* name; } kernels[256];
+static int n_kernels = 0;
+const char* fake_last_kernel = "";
+
+static int launch(const void* f, void* stream) {
   if (stream == (void*)kStreamDevice1 && fake_device != 1) {
     ++fake_refused;
     return last_error = kInvalidResourceHandle;
   }
   ++fake_launches;
+  for (int i = 0; i < n_kernels; ++i)
+    if (kernels[i].f == f) fake_last_kernel = kernels[i].name;
   return 0;
 }
 static void* pushed_stream;
@@ -99,16 +121,22 @@ int __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* m, void** s) {
 }
 int __cudaGetKernel(void** k, const void* f) { *k = (void*)f; return 0; }
 int __cudaLaunchKernel(void* k, dim3 g, dim3 b, void** a, size_t m, void* s) {
-  (void)k; (void)g; (void)b; (void)a; (void)m;
-  return launch(s);
+  (void)g; (void)b; (void)a; (void)m;
+  return launch(k, s);
 }
 typedef struct { dim3 grid, block; size_t smem; void* stream; void* attrs; unsigned n; } Config;
-int cudaLaunchKernelExC(const Config* c, const void* f, void** a) { (void)f; (void)a; return launch(c->stream); }
+int cudaLaunchKernelExC(const Config* c, const void* f, void** a) { (void)a; return launch(f, c->stream); }
 
 void** __cudaRegisterFatBinary(void* p) { (void)p; static void* h; return &h; }
 void __cudaRegisterFatBinaryEnd(void** h) { (void)h; }
 void __cudaUnregisterFatBinary(void** h) { (void)h; }
-void __cudaRegisterFunction(void) {}
+void __cudaRegisterFunction(void** h, const char* f, char* device_f, const char* name) {
+  (void)h; (void)device_f;
+  if (n_kernels < 256) {
+    kernels[n_kernels].f = f;
+    kernels[n_kernels++].name = name;
+  }
+}
 void __cudaRegisterVar(void) {}
 
 /* not reached by these tests */

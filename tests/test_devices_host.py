@@ -16,6 +16,7 @@ import ctypes as C, sys
 lib = C.CDLL(sys.argv[1])
 fake = C.CDLL("libcudart.so.13")
 word = lambda name: C.c_int.in_dll(fake, name)
+last_kernel = lambda name: name.encode() in C.c_char_p.in_dll(fake, "fake_last_kernel").value
 from paper_2605_07083_gb300 import pic, workloads as W
 for name, (res, args) in pic.ENTRY_POINTS.items():
     getattr(lib, name).restype, getattr(lib, name).argtypes = res, args
@@ -61,11 +62,29 @@ n = C.c_int64()
 copies = word("fake_copies").value
 assert lib.pic_inject(h, 0, 0, 512, a[0], a[1], a[4], a[3], 1) == 0
 assert (word("fake_copies").value == copies) == {direct}
-# the counts come from kernels, which the stand-in does not run: no particles
-# to copy, and one launch either way
-launches = word("fake_launches").value
 assert lib.pic_get_state(h, 0, 0, *a, 512, C.byref(n), 1) == 0
-assert word("fake_launches").value == launches + 1
+assert last_kernel("k_state_copy" if {direct} else "k_read")
+''')
+
+
+@pytest.mark.parametrize("elements,offset,direct", [(512, 0, True), (511, 0, False), (600, 88, True),
+                                                    (600, 89, False)])
+def test_a_count_beyond_the_array_is_not_read_by_kernels(run, elements, offset, direct):
+    """512 particles from (to) an array with `elements` of them, from `offset`
+    on: past its end cudaMemcpyAsync is asked, which refuses what does not fit
+    (the stand-in copies: the memory behind the array is there)."""
+    run(f'''
+h = create()
+whole = (C.c_float * 1024)()
+fake.fake_array(whole, 4 * {elements}, {DEVICE}, 1)
+short = C.byref(whole, 4 * {offset})
+a = [array(512, {DEVICE}, 1) for _ in range(3)]
+copies = word("fake_copies").value
+assert lib.pic_inject(h, 0, 0, 512, a[0], short, a[1], a[2], 1) == 0
+assert (word("fake_copies").value == copies) == {direct}
+n = C.c_int64()
+assert lib.pic_get_state(h, 0, 0, a[0], short, a[1], a[2], None, 512, C.byref(n), 1) == 0
+assert last_kernel("k_state_copy" if {direct} else "k_read")
 ''')
 
 
