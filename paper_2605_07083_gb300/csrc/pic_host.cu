@@ -1290,7 +1290,7 @@ int pic_profile_steps(pic_handle* h, int64_t n_steps, pic_profile* out) {
       launch_sort(h);
       cudaEventRecord(e[4], h->stream);
       sorted[i] = 1;
-      out->launches += 3;
+      out->launches += kSortKernels;
     }
   }
   cudaEventRecord(t1, h->stream);

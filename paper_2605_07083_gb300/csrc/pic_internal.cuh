@@ -198,6 +198,7 @@ struct DevState {
 };
 
 struct SortGrid { int chunks, tiles, copies; };    // blocks per segment of the sort's kernels
+constexpr int kSortKernels = 5;          // launches of a sort (sort_launch)
 
 // Is the state after step n a profile sample?  (Sec. 3 late-time averages:
 // steps n >= window_start with (n - window_start) a multiple of the period.)
