@@ -210,9 +210,11 @@ int pic_step(pic_handle* h, int64_t n_steps);
  * would launch, so that the call itself only launches (the first pic_step
  * that needs a graph otherwise captures it, a one-time host cost of about a
  * millisecond per 64 steps).  Runs no step; the charge and field of an
- * injected or loaded state are computed first, as pic_step would.  Returns a
- * sticky error seen earlier, PIC_EINVAL for a null handle or n_steps < 0, or
- * PIC_ECUDA if a capture fails. */
+ * injected or loaded state are computed first, as pic_step would.  Later calls
+ * of as many steps capture nothing either, but for a periodic sort without
+ * profile samples: there a call from another place in the sort period may.
+ * Returns a sticky error seen earlier, PIC_EINVAL for a null handle or
+ * n_steps < 0, or PIC_ECUDA if a capture fails. */
 int pic_prepare_steps(pic_handle* h, int64_t n_steps);
 
 /* Same steps as pic_step, launched one by one with CUDA events around each

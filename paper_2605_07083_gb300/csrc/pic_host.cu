@@ -1222,11 +1222,30 @@ static int plan_stretch(pic_handle* h, int64_t n_steps, int64_t step, bool run) 
   return PIC_OK;
 }
 
+// Captures the graphs of at most n_steps steps that are not there yet.
+static int capture_up_to(pic_handle* h, int64_t n_steps) {
+  const int len = graph_unit(h);
+  if (len <= 0) return PIC_OK;
+  if (h->graphs.empty() || h->graphs[0].first != len) plan_graphs(h);
+  for (auto& g : h->graphs)
+    if (g.first <= n_steps && !g.second) {
+      int rc = build_graph(h, g.first, &g.second);
+      if (rc != PIC_OK) return rc;
+    }
+  return PIC_OK;
+}
+
 // The plan of pic_step(n) from the current step: stretches between sampled
-// steps, and those by themselves.
+// steps, and those by themselves.  Where the stretches fall depends on the step
+// the call starts from, so a preparation (run not set) captures every graph
+// that a stretch of up to n steps can need, not those of this start alone.
 static int step_plan(pic_handle* h, int64_t n_steps, bool run) {
   int64_t left = n_steps, step = h->host_step;
   const bool split = h->st.prof_period > 0 && !h->profile_each;
+  if (split && !run) {
+    const int64_t gap = std::max<int64_t>(h->st.prof_period - 1, steps_to_sample(h, step));
+    return capture_up_to(h, std::min(n_steps, gap));
+  }
   while (left > 0) {
     const int64_t gap = split ? steps_to_sample(h, step) : left;
     const int64_t m = std::max<int64_t>(1, std::min(left, gap));

@@ -2,7 +2,7 @@
  * side of the library: memory is the host's, launches run nothing.  It keeps
  * what the tests look at -- the current device, launches on a stream of
  * another device (refused, as the runtime does), copies, the device on which
- * each kernel attribute was set -- and answers pointer queries from a table
+ * each kernel attribute was set, captured and launched graphs -- and answers pointer queries from a table
  * that the test fills in. */
 #include <stddef.h>
 #include <stdint.h>
@@ -139,6 +139,12 @@ void __cudaRegisterFunction(void** h, const char* f, char* device_f, const char*
 }
 void __cudaRegisterVar(void) {}
 
+int fake_captures = 0, fake_graph_launches = 0;
+int cudaStreamBeginCapture(void* s, int mode) { (void)s; (void)mode; ++fake_captures; return 0; }
+int cudaStreamEndCapture(void* s, void** g) { (void)s; *g = (void*)0x3000; return 0; }
+int cudaGraphInstantiate(void** x, void* g, unsigned long long f) { (void)g; (void)f; *x = (void*)0x4000; return 0; }
+int cudaGraphLaunch(void* x, void* s) { (void)x; (void)s; ++fake_graph_launches; return 0; }
+
 /* not reached by these tests */
 int cudaEventCreate(void** e) { *e = NULL; return kInvalidValue; }
 int cudaEventDestroy(void* e) { (void)e; return 0; }
@@ -151,8 +157,4 @@ int cudaGraphConditionalHandleCreate(void) { return kInvalidValue; }
 int cudaGraphCreate(void) { return kInvalidValue; }
 int cudaGraphDestroy(void) { return 0; }
 int cudaGraphExecDestroy(void) { return 0; }
-int cudaGraphInstantiate(void) { return kInvalidValue; }
-int cudaGraphLaunch(void) { return kInvalidValue; }
-int cudaStreamBeginCapture(void) { return kInvalidValue; }
 int cudaStreamBeginCaptureToGraph(void) { return kInvalidValue; }
-int cudaStreamEndCapture(void) { return kInvalidValue; }

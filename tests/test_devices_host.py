@@ -1,5 +1,6 @@
-"""What the library's host side does in a process with two devices, on a
-stand-in for the CUDA runtime (fake_cudart.c): no GPU, nothing is launched.
+"""What the library's host side does, in a process with two devices among other
+things, on a stand-in for the CUDA runtime (fake_cudart.c): no GPU, nothing is
+launched.
 Each case runs in a process of its own, which loads the library against the
 stand-in."""
 import os
@@ -121,4 +122,27 @@ for device in (0, 1, 1, 0):
     if device == 1:
         assert seen[1] == seen[0] > 0
 assert list(counts) == seen
+''')
+
+
+@pytest.mark.parametrize("window,period,steps", [(0, 100, 50), (70, 100, 130), (1000, 33, 250),
+                                                 (0, 100, 3)])
+def test_prepared_steps_capture_nothing_at_any_phase_of_the_samples(run, window, period, steps):
+    """Sampled steps run by themselves, so the stretches between them start
+    anywhere: after one preparation no later call of as many steps captures."""
+    run(f'''
+h = C.c_void_p()
+word("fake_device").value = 1
+p = dict(W.single_diode_small(), capacity=(4096,) * 3, window_start={window})
+cfg = pic.make_config(p)
+assert lib.pic_create(C.byref(cfg), 1, C.c_void_p(0x1000), None, C.byref(h)) == 0
+t = pic.PicTuning(size=C.sizeof(pic.PicTuning), wait_polls=5)   # three kernels a step
+assert lib.pic_tune(h, C.byref(t)) == 0
+assert lib.pic_set_profile_period(h, {period}) == 0
+assert lib.pic_prepare_steps(h, {steps}) == 0
+captures = word("fake_captures").value
+for _ in range(40):
+    assert lib.pic_step(h, {steps}) == 0
+assert word("fake_graph_launches").value > 0 and captures > 0
+assert word("fake_captures").value == captures
 ''')
