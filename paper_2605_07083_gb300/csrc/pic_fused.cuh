@@ -704,7 +704,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
         if (lane < n_item) fused_dead(st, ic, item_sp, off_of(item_sp), dd[item_part + kp * lane], d);
       } else {
         FusedDead sum{0, 0, 0.0, 0.0};           // lane v < 16: virtual warp v
-        for (int v = 0; v < kPostThreads / 32; ++v) {
+        const int nv = min(kPostThreads / 32, (n_item + 31) >> 5);   // the others hold zeros
+        for (int v = 0; v < nv; ++v) {
           FusedDead e{0, 0, 0.0, 0.0};
           for (int t = 32 * v + lane; t < n_item; t += kPostThreads)
             fused_dead(st, ic, item_sp, off_of(item_sp), dd[item_part + kp * t], e);
