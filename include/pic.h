@@ -225,6 +225,12 @@ int pic_profile_steps(pic_handle* h, int64_t n_steps, pic_profile* out);
 /* Window tallies and Eq. 1-8 diagnostics of one instance.  Synchronises. */
 int pic_diagnostics(pic_handle* h, int instance, pic_diag* out);
 
+/* How many of the handle's steps so far (modulo 2^32) ran in the kernel that
+ * takes whole steps of small diodes, a thread-block cluster each; the others
+ * ran as three kernels.  pic_step chooses on the device; the results are the
+ * same either way.  Synchronises. */
+int pic_fused_steps(pic_handle* h, int64_t* steps);
+
 /* Copy out the live particles of one species.  cap = room in the buffers;
  * *n receives the live count (PIC_ECAPACITY if cap < *n, nothing copied).
  * Any buffer may be NULL.  Synchronises. */

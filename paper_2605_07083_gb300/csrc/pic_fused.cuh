@@ -806,6 +806,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
       dyn->step = S.step;
       dyn->next_id = S.base_id;
       dyn->pushed += S.pushed;
+      st.post[inst].fused_steps += (uint32_t)n_steps;
       dyn->win_steps += S.win_steps;
       dyn->emitted += S.emitted;
       dyn->replenished += S.replenished;

@@ -1350,6 +1350,16 @@ int pic_diagnostics(pic_handle* h, int instance, pic_diag* out) {
   return flags_of(h);
 }
 
+int pic_fused_steps(pic_handle* h, int64_t* steps) {
+  if (!h || !steps) return PIC_EINVAL;
+  OnDevice on(h);
+  k_read<<<1, 256, 0, h->stream>>>(h->st, 0, h->rb);
+  int rc = read_done(h);
+  if (rc != PIC_OK) return rc;
+  *steps = (int64_t)h->rb->fused_steps;
+  return flags_of(h);
+}
+
 int pic_get_state(pic_handle* h, int instance, int species, float* z, float* vx, float* vy,
                   float* vz, uint32_t* id, int64_t cap, int64_t* n, int on_device) {
   if (!h || !n || instance < 0 || instance >= h->n_inst || species < 0 || species > 2)

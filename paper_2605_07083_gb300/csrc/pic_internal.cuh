@@ -119,7 +119,7 @@ struct InstDyn {
 struct PostScratch {
   int D[3], N[3];
   uint32_t base_id;
-  int32_t pad;
+  uint32_t fused_steps;              // steps that k_fused has run
   long long step;
   long long cnt[3][kMaxParts][2];    // per species, per k_mid list block, per electrode
   double ke[3][kMaxParts][2];
@@ -132,7 +132,7 @@ struct Readback {
   int err;                 // error bits of all diodes
   int bad;                 // pic_inject: blocks that saw a z outside [0, L)
   int count[3];            // live particles of the diode
-  int pad;
+  uint32_t fused_steps;    // PostScratch
   InstDyn dyn;
 };
 constexpr size_t kReadNodes = 1024;

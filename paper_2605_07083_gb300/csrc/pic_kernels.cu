@@ -1208,6 +1208,7 @@ __global__ void k_read(DevState st, int inst, Readback* out) {
   int* dst = reinterpret_cast<int*>(&out->dyn);
   for (int w = threadIdx.x; w < (int)(sizeof(InstDyn) / 4); w += blockDim.x) dst[w] = src[w];
   if (threadIdx.x < 3) out->count[threadIdx.x] = st.seg_count[3 * inst + threadIdx.x];
+  if (threadIdx.x == 0) out->fused_steps = st.post[inst].fused_steps;
 }
 
 // errors and the diode's fixed-point charge

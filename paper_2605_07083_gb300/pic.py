@@ -104,6 +104,7 @@ ENTRY_POINTS = {
     "pic_prepare_steps": (C.c_int, [_P, C.c_int64]),
     "pic_profile_steps": (C.c_int, [_P, C.c_int64, C.POINTER(PicProfile)]),
     "pic_diagnostics": (C.c_int, [_P, C.c_int, C.POINTER(PicDiag)]),
+    "pic_fused_steps": (C.c_int, [_P, C.POINTER(C.c_int64)]),
     "pic_get_state": (C.c_int, [_P, C.c_int, C.c_int, _P, _P, _P, _P, _P, C.c_int64,
                                 C.POINTER(C.c_int64), C.c_int]),
     "pic_get_rho_fixed": (C.c_int, [_P, C.c_int, _P, C.c_int64]),
@@ -282,6 +283,12 @@ def pic_diagnostics(h, instance=0, check=True) -> dict:
     return out
 
 
+def pic_fused_steps(h) -> int:
+    n = C.c_int64()
+    _check(load().pic_fused_steps(h, C.byref(n)), "pic_fused_steps")
+    return n.value
+
+
 def pic_get_state(h, instance, species, device=False):
     lib = load()
     n = C.c_int64()
@@ -442,6 +449,10 @@ class Diode:
 
     def diagnostics(self, instance=0, check=True):
         return pic_diagnostics(self._h, instance, check)
+
+    def fused_steps(self):
+        """Steps so far that ran in the one-kernel form (small diodes)."""
+        return pic_fused_steps(self._h)
 
     def state(self, species, instance=0, device=False):
         return pic_get_state(self._h, instance, species, device)
