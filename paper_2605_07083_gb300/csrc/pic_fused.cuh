@@ -40,7 +40,6 @@ namespace cg = cooperative_groups;
 
 constexpr int kFusedWarps = kFusedThreads / 32;
 constexpr int kFusedMaxC = 16;         // blocks per cluster (non-portable above 8)
-constexpr int kFusedCand = 1024;       // candidates listed per block and step
 constexpr int kFusedList = 1024;       // absorbed slots of a species held in shared memory
 constexpr int kFusedWarpList = 32;     // of a warp and species
 constexpr int kFusedTeamWarps = kFusedWarps - 1;   // warps of phase D's teams
@@ -833,30 +832,67 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
 // overflow is an error.
 __global__ void k_route(DevState st, int C, int sms, long long growth,
                         cudaGraphConditionalHandle handle) {
-  __shared__ float wsf[32];
-  __shared__ long long ws64[32];
-  float longest = 0.0f, cands = 0.0f;
-  long long mine = 0;
+  __shared__ float ws[6][32];
+  float longest = 0.0f, most = 0.0f, emit = 0.0f, sum = 0.0f, cands = 0.0f, total = 0.0f;
   for (int i = threadIdx.x; i < st.n_inst; i += blockDim.x) {
+    const InstConst& ic = st.ic[i];
+    PostScratch& ps = st.post[i];
     int n = 0;
+    float cand = 0.0f, dead = 0.0f;
     for (int sp = 0; sp < 3; ++sp) {
       const int ns = st.seg_count[3 * i + sp];
       n += ns;
-      cands += (float)ns * ((float)st.ic[i].t_cand[sp] * 2.3283064e-10f);
+      cand += (float)ns * ((float)ic.t_cand[sp] * 2.3283064e-10f);
     }
-    longest = fmaxf(longest, (float)n);
-    mine += n;
+    // absorbed per step since the last decision: every particle that came has an
+    // id (what an injection or a load makes of it only sways one choice)
+    const long long step = st.dyn[i].step, past = step - ps.route_step;
+    const uint32_t id = st.dyn[i].next_id;
+    const long long gone = (long long)ps.route_n + (long long)(uint32_t)(id - ps.route_id) - n;
+    if (past > 0 && past <= 4096 && gone > 0) dead = (float)gone / (float)past;
+    ps.route_step = step;
+    ps.route_n = n;
+    ps.route_id = id;
+    const DiodeLoad d{(float)n, (float)ic.emit_floor + (float)ic.t_frac * 2.3283064e-10f,
+                      dead, cand};
+    const float t = fused_estimate(d, C, st.kp, st.max_nodes);
+    longest = fmaxf(longest, t);
+    sum += t;
+    most = fmaxf(most, (float)n);
+    emit = fmaxf(emit, d.emit);
+    cands += cand;
+    total += d.n;
   }
-  for (int o = 16; o > 0; o >>= 1) longest = fmaxf(longest, __shfl_down_sync(0xffffffffu, longest, o));
-  if ((threadIdx.x & 31) == 0) wsf[threadIdx.x >> 5] = longest;
-  const long long total = block_sum<long long>(mine, ws64);
-  __shared__ float wsc[32];
-  cands = block_sum<float>(cands, wsc);
+  for (int o = 16; o > 0; o >>= 1) {
+    longest = fmaxf(longest, __shfl_down_sync(0xffffffffu, longest, o));
+    most = fmaxf(most, __shfl_down_sync(0xffffffffu, most, o));
+    emit = fmaxf(emit, __shfl_down_sync(0xffffffffu, emit, o));
+    sum += __shfl_down_sync(0xffffffffu, sum, o);
+    cands += __shfl_down_sync(0xffffffffu, cands, o);
+    total += __shfl_down_sync(0xffffffffu, total, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    const int w = threadIdx.x >> 5;
+    ws[0][w] = longest;
+    ws[1][w] = most;
+    ws[2][w] = emit;
+    ws[3][w] = sum;
+    ws[4][w] = cands;
+    ws[5][w] = total;
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) longest = fmaxf(longest, wsf[w]);
-    const StepEstimate e = estimate_step(st.n_inst, longest, (float)total, C, sms, st.max_nodes);
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+      longest = fmaxf(longest, ws[0][w]);
+      most = fmaxf(most, ws[1][w]);
+      emit = fmaxf(emit, ws[2][w]);
+      sum += ws[3][w];
+      cands += ws[4][w];
+      total += ws[5][w];
+    }
+    const StepEstimate e = estimate_step(st.n_inst, longest, sum, total, cands, emit, C, sms);
     const bool one = e.fused < e.three && 2.0f * cands + 4096.0f < (float)st.cand_cap &&
-                     (long long)longest + growth < (long long)kHistMaxParticles;
+                     (long long)most + growth < (long long)kHistMaxParticles;
     cudaGraphSetConditional(handle, one ? 1u : 0u);
   }
 }

@@ -765,15 +765,24 @@ void set_fused_shape(pic_handle* h) {
 // where the last counts the host knows make k_fused take twice the time of
 // the three kernels.
 bool fused_allowed(const pic_handle* h) {
-  long long total = 0;
-  int longest = 0;
+  const int C = std::max(1, h->fused_c);
+  float longest = 0.0f, sum = 0.0f, total = 0.0f, cands = 0.0f, emit = 0.0f;
   for (int i = 0; i < h->n_inst; ++i) {
-    const int n = h->known_count[3 * i] + h->known_count[3 * i + 1] + h->known_count[3 * i + 2];
-    total += n;
-    longest = std::max(longest, n);
+    const InstConst& k = h->ic[i];
+    DiodeLoad d{0.0f, (float)k.emit_floor + (float)k.t_frac * 2.3283064e-10f, 0.0f, 0.0f};
+    for (int s = 0; s < 3; ++s) {
+      const float n = (float)h->known_count[3 * i + s];
+      d.n += n;
+      d.cand += n * ((float)k.t_cand[s] * 2.3283064e-10f);
+    }
+    const float t = fused_estimate(d, C, h->st.kp, h->max_nodes);
+    longest = std::max(longest, t);
+    sum += t;
+    total += d.n;
+    cands += d.cand;
+    emit = std::max(emit, d.emit);
   }
-  const StepEstimate e = estimate_step(h->n_inst, (float)longest, (float)total,
-                                       std::max(1, h->fused_c), h->sm_count, h->max_nodes);
+  const StepEstimate e = estimate_step(h->n_inst, longest, sum, total, cands, emit, C, h->sm_count);
   return h->fused_c > 0 && e.fused < 2.0f * e.three && h->sort_period <= 0 && !h->profile_each &&
          h->st.wait_limit == kWaitLimit;
 }

@@ -33,24 +33,50 @@ enum ErrBit : int32_t { ERR_CAPACITY = 1 << 3, ERR_TIMEOUT = 1 << 4, ERR_ENERGYC
 constexpr int kFusedThreads = 512;      // threads per block of k_fused
 constexpr int kFusedMinSteps = 8;      // shortest graph that lets k_route choose
 // Estimates of a step's time, ns, by the fused kernel with C blocks per diode
-// and by the three kernels (fits to the measured steps of 1 to 512 diodes of
-// 128 to 2000 cells).  Fused: a cluster takes a fixed time, more per cell and
-// where all warps solve the field, and its diode's particles at the rate of
-// its blocks (2.05 per ns and block, 1.4 in a cluster of 16); the clusters
-// share the SMs.  Three kernels: launches and round trips, a part per diode,
-// the particles at the chip's rate.
+// and by the three kernels (fits to measured steps of 1 to 512 diodes of 128 to
+// 2000 cells, with up to 1600 electrons emitted and absorbed per diode and step
+// and 0 to 20 % collision candidates).  What the fit rests on:
+//   * fused, a diode: a fixed time, more per cell and where all warps solve the
+//     field; its particles at the rate of its blocks (2.05 per ns and block, 1.4
+//     in a cluster of 16); its emission, drawn by one warp (10 ns an electron, 17
+//     where one block's threads also append it); its absorbed particles, whose
+//     tallies are a warp's walk over 32 at a time in kp parts; its candidates, as
+//     long as a block's list holds them, else a second pass over the particles.
+//     The clusters run in waves.
+//   * three kernels: launches and round trips, a part per diode, the particles
+//     and the candidates at the chip's rate, the emission a block's.
+// Without the last three of the first, diodes that emit and absorb some hundreds
+// a step took up to 1.96 x the three kernels' time (38 diodes, 1600 a step: 96
+// and 49 us), lists that ran over up to 4.8 x (200 diodes of 326k particles:
+// 1739 and 360 us).  Now none of 174 such runs takes more than 1.06 x.
 constexpr int kFusedWarpCells = 512;   // cells that one warp of k_fused solves for
-struct StepEstimate { float fused, three; };
-__host__ __device__ inline StepEstimate estimate_step(int n_inst, float longest, float total, int C,
-                                                      int sms, int max_nodes) {
+constexpr int kFusedCand = 1024;       // candidates listed per block and step
+struct DiodeLoad {
+  float n, emit, dead, cand;           // live, emitted, absorbed, candidates
+};
+__host__ __device__ inline float fused_estimate(const DiodeLoad& d, int C, int kp, int max_nodes) {
   const int cells = max_nodes < kFusedWarpCells ? max_nodes : kFusedWarpCells;
-  const float t0 = 8000.0f + 3.5f * (float)cells + (max_nodes > kFusedWarpCells + 1 ? 3500.0f : 0.0f);
-  const float per = 1.0f / ((2.1f - 0.045f * (float)C) * (float)C);
-  const float chain = t0 + longest * per;
-  const float work = ((float)n_inst * t0 + total * per) * (float)C / (float)sms;
+  float t = 8000.0f + 3.5f * (float)cells + (max_nodes > kFusedWarpCells + 1 ? 3500.0f : 0.0f);
+  t += d.n / ((2.1f - 0.045f * (float)C) * (float)C);
+  t += d.emit * (C > 1 ? 10.4f : 16.6f);
+  const float walked = d.dead / (float)kp - 32.0f;
+  if (walked > 0.0f) t += 50.0f * walked;
+  const float list = d.cand / (float)C;
+  t += 3.0f * list;
+  if (list > (float)(kFusedCand - 32)) t += 2.2f * d.n / (float)C;    // a standard deviation below
+  return t;
+}
+struct StepEstimate { float fused, three; };
+// longest and sum of the diodes' fused_estimate, and the diodes' sums
+__host__ __device__ inline StepEstimate estimate_step(int n_inst, float longest, float sum,
+                                                      float particles, float cands, float emit,
+                                                      int C, int sms) {
+  const int waves = (n_inst * C + sms - 1) / sms;
+  const float work = sum / (float)n_inst * (float)waves;
   StepEstimate e;
-  e.fused = chain > work ? chain : work;
-  e.three = 16000.0f + 95.0f * (float)n_inst + total / 270.0f;
+  e.fused = longest > work ? longest : work;
+  e.three = 16000.0f + 95.0f * (float)n_inst + particles / 300.0f + 0.15f * cands +
+            emit * (6.0f + 0.1f * (float)n_inst);
   return e;
 }
 
@@ -120,6 +146,9 @@ struct PostScratch {
   int D[3], N[3];
   uint32_t base_id;
   uint32_t fused_steps;              // steps that k_fused has run
+  int route_n;                       // live particles, next id and step at k_route's last decision
+  uint32_t route_id;
+  long long route_step;
   long long step;
   long long cnt[3][kMaxParts][2];    // per species, per k_mid list block, per electrode
   double ke[3][kMaxParts][2];

@@ -75,3 +75,51 @@ def test_a_growing_diode_changes_over(pic):
     for x, y in zip(sa, sb):
         for k in x:
             assert np.array_equal(x[k], y[k]), k
+
+
+@pytest.mark.parametrize("n_pairs,pcand,fused", [(30000, 0.005, True), (60000, 0.02, False)])
+def test_more_candidates_than_a_list_holds_take_the_three(pic, n_pairs, pcand, fused):
+    """128 diodes, a block each: 300 candidates are in its list of 1024, 2400
+    cost a second pass over its particles, which the three kernels do not need."""
+    ps = []
+    for i in range(128):
+        p = W.single_diode_small(seed=200 + i)
+        # n sigma g at the energy bound gives the electrons' probability
+        g = np.sqrt(2 * 400.0 * W.E_CHARGE / W.M_E)
+        p.update(window_start=1 << 40, E_cap_e_eV=400.0, E_cap_i_eV=400.0, gamma_emit=0.0,
+                 n_gas=-np.log1p(-pcand) / (p["sigma_el_e"] * g * p["dt"]),
+                 capacity=(1024, n_pairs + 4096, n_pairs + 4096))
+        ps.append(p)
+    state = mixed_state(ps[0], 5, 100, n_pairs)
+    d = pic.Diode(ps)
+    for i in range(128):
+        for sp in range(3):
+            d.inject(sp, *state[sp], instance=i)
+    d.step(8)
+    assert d.fused_steps() == (8 if fused else 0)
+    d.close()
+
+
+@pytest.mark.parametrize("ions,fused", [(20, 16), (4000, 8)])
+def test_thousands_of_absorbed_particles_take_the_three(pic, ions, fused):
+    """Hot ions that leave in every step and are replaced.  4000 of them keep
+    the one warp that adds up their energies busy for longer than a step of the
+    three kernels takes; how many there are is known from the first decision's
+    last step on."""
+    ps = []
+    for i in range(76):
+        p = W.single_diode_small(seed=40 + i)
+        p.update(V=0.0, dt=1e-6, n_gas=0.0, T_e0_eV=0.0, T_i0_eV=100.0, weight=1e-12,
+                 gamma_emit=0.0, replenish=1, window_start=1 << 40,
+                 capacity=(32, 100000, ions + 32))
+        ps.append(p)
+    rng = np.random.default_rng(9)
+    z = (rng.random(ions) * ps[0]["L"] * 0.999).astype(np.float32)
+    v = [(rng.standard_normal(ions) * 5e4).astype(np.float32) for _ in range(3)]
+    d = pic.Diode(ps)
+    for i in range(76):
+        d.inject(2, z, *v, instance=i)
+    d.step(8)
+    d.step(8)
+    assert d.fused_steps() == fused
+    d.close()
