@@ -236,10 +236,15 @@ def pic_create(configs, stream=None, allocator=None):
 
 
 def pic_inject(h, instance, species, z, vx, vy, vz):
-    """z, vx, vy, vz: numpy float32 arrays (host) or CUDA float32 tensors."""
+    """z, vx, vy, vz: numpy float32 arrays (host) or CUDA float32 tensors, read
+    on the handle's stream: work that fills them on another stream has to be done."""
     on_dev = hasattr(z, "is_cuda") and z.is_cuda
     if on_dev:
-        keep = [t.float().contiguous() for t in (z, vx, vy, vz)]   # alive across the call
+        given = (z, vx, vy, vz)
+        keep = [t.float().contiguous() for t in given]   # alive across the call
+        if any(k is not t for k, t in zip(keep, given)):
+            import torch
+            torch.cuda.current_stream(z.device).synchronize()   # copies made here, on that stream
         ptrs = [t.data_ptr() for t in keep]
         n = keep[0].numel()
     else:
