@@ -305,6 +305,9 @@ def pic_get_state(h, instance, species, device=False):
         import torch
         bufs = [torch.empty(cnt, dtype=torch.float32, device="cuda") for _ in range(4)]
         ids = torch.empty(cnt, dtype=torch.int32, device="cuda")
+        # the blocks may still be in use by work on this stream; the handle's
+        # stream, on which they are written, does not wait for it
+        torch.cuda.current_stream().synchronize()
         ptrs = [b.data_ptr() for b in bufs] + [ids.data_ptr()]
     else:
         bufs = [np.empty(cnt, np.float32) for _ in range(4)]

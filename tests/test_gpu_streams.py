@@ -42,3 +42,27 @@ def test_converted_arrays_are_complete_when_they_are_read(pic, form):
     for k, a in zip(("z", "vx", "vy", "vz"), state):
         assert np.array_equal(got[k], a), k
     d.close()
+
+
+def test_state_tensors_are_not_written_while_their_memory_is_in_use(pic):
+    """Freed tensors whose last writes are still queued behind other work on
+    the current stream: their memory comes back as the state's tensors, which
+    must be written after those writes."""
+    import torch
+    p = W.single_diode_small(seed=72)
+    d = pic.Diode(p)
+    d.inject(0, *mixed_state(p, 73, 4001, 10)[0])
+    want = d.state(0)
+    d.state(0, device=True)                # (a kernel's first launch may wait for the GPU)
+    n = want["z"].size
+    old = [torch.zeros(n, device="cuda") for _ in range(64)]
+    torch.cuda.synchronize()
+    torch.cuda._sleep(100_000_000)
+    for t in old:
+        t.fill_(-1.0)
+    del old, t
+    got = d.state(0, device=True)
+    torch.cuda.synchronize()
+    for k in ("z", "vx", "vy", "vz"):
+        assert np.array_equal(got[k].cpu().numpy(), want[k]), k
+    d.close()
