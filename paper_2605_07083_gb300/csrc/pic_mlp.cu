@@ -45,9 +45,9 @@ constexpr int kSms = 152;                    // tiles are kept to one wave while
 template <int TS>
 struct Tile {
   static constexpr int kRow = TS + 4;        // floats per row of an activation array
-  static constexpr int kSpw = 4;             // samples per warp
-  static constexpr int kSg = TS / kSpw;      // groups of that many
+  static constexpr int kSg = TS / 4;         // groups of the four samples that a warp takes
   static constexpr int kSplit = kWarps / kSg;    // warps that share a group's contraction
+  static_assert(kSplit > 1, "the partial sums of a group go through shared memory");
 };
 
 template <int TS>
@@ -57,7 +57,7 @@ struct Smem {
   float b1[H], b2[H], b3[H], b4[OUT];
   float a0[IN][Tile<TS>::kRow];
   float dy[OUT][Tile<TS>::kRow];
-  float part[Tile<TS>::kSplit][Tile<TS>::kSplit > 1 ? H : 1][Tile<TS>::kRow];   // partial sums
+  float part[Tile<TS>::kSplit][H][Tile<TS>::kRow];   // partial sums
   float ypart[kThr / TS][TS];                // output-layer partial sums
   float a1[H][Tile<TS>::kRow], a2[H][Tile<TS>::kRow];
 };
@@ -190,21 +190,18 @@ __device__ __forceinline__ void load_tile(Smem<TS>& S, const float* __restrict__
 template <int TS>
 __device__ __forceinline__ void product_forward(const __nv_bfloat16 (*wt)[kWRow],
                                                 const float (*in)[Tile<TS>::kRow], int sg, int part,
-                                                f2 (&acc)[4][Tile<TS>::kSpw / 2]) {
-  constexpr int kLen = H / Tile<TS>::kSplit, kSpw = Tile<TS>::kSpw;
+                                                f2 (&acc)[4][2]) {
+  constexpr int kLen = H / Tile<TS>::kSplit;
   const int lane = threadIdx.x & 31, c0 = part * kLen;
 #pragma unroll 8
   for (int c = c0; c < c0 + kLen; ++c) {
     const uint2 wv = *reinterpret_cast<const uint2*>(&wt[c][4 * lane]);
     const f2 d[4] = {dup_lo(wv.x), dup_hi(wv.x), dup_lo(wv.y), dup_hi(wv.y)};
+    const ulonglong2 av = *reinterpret_cast<const ulonglong2*>(&in[c][4 * sg]);
 #pragma unroll
-    for (int p = 0; p < kSpw / 4; ++p) {
-      const ulonglong2 av = *reinterpret_cast<const ulonglong2*>(&in[c][kSpw * sg + 4 * p]);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        acc[r][2 * p] = fma2(d[r], av.x, acc[r][2 * p]);
-        acc[r][2 * p + 1] = fma2(d[r], av.y, acc[r][2 * p + 1]);
-      }
+    for (int r = 0; r < 4; ++r) {
+      acc[r][0] = fma2(d[r], av.x, acc[r][0]);
+      acc[r][1] = fma2(d[r], av.y, acc[r][1]);
     }
   }
 }
@@ -252,54 +249,40 @@ __device__ __forceinline__ void activate4(const float (&z)[4], float* act, float
 }
 
 // a hidden layer: out = gelu(W in + b), slopes for training, for the first
-// `live` samples of the tile (rounded up to a group).  A contraction split
-// over warps is summed part by part after a barrier.
+// `live` samples of the tile (rounded up to a group).  The contraction is split
+// over kSplit warps and summed part by part after a barrier.
 template <int TS, bool kGrad>
 __device__ __forceinline__ void hidden_layer(Smem<TS>& S, const __nv_bfloat16 (*wt)[kWRow],
                                              const float* b, const float (*in)[Tile<TS>::kRow],
                                              float (*out)[Tile<TS>::kRow],
                                              float (*slope)[Tile<TS>::kRow], int live) {
-  constexpr int kSpw = Tile<TS>::kSpw, kSg = Tile<TS>::kSg;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int sg = warp % kSg, part = warp / kSg;
-  f2 acc[4][kSpw / 2];
+  const int sg = warp % Tile<TS>::kSg, part = warp / Tile<TS>::kSg;
+  if (4 * sg < live) {
+    f2 acc[4][2];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const float b0 = part == 0 ? b[4 * lane + r] : 0.0f;
-#pragma unroll
-    for (int p = 0; p < kSpw / 2; ++p) acc[r][p] = pack2(b0, b0);
-  }
-  if (kSpw * sg < live) {
+    for (int r = 0; r < 4; ++r) {
+      const float b0 = part == 0 ? b[4 * lane + r] : 0.0f;
+      acc[r][0] = acc[r][1] = pack2(b0, b0);
+    }
     product_forward<TS>(wt, in, sg, part, acc);
 #pragma unroll
     for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int p = 0; p < kSpw / 4; ++p) {
-        const int j = 4 * lane + r, at = kSpw * sg + 4 * p;
-        if (Tile<TS>::kSplit == 1) {
-          const float z[4] = {lo2(acc[r][2 * p]), hi2(acc[r][2 * p]), lo2(acc[r][2 * p + 1]),
-                              hi2(acc[r][2 * p + 1])};
-          activate4<kGrad>(z, &out[j][at], kGrad ? &slope[j][at] : nullptr);
-        } else {
-          *reinterpret_cast<ulonglong2*>(&S.part[part][j][at]) =
-              make_ulonglong2(acc[r][2 * p], acc[r][2 * p + 1]);
-        }
-      }
+      *reinterpret_cast<ulonglong2*>(&S.part[part][4 * lane + r][4 * sg]) =
+          make_ulonglong2(acc[r][0], acc[r][1]);
   }
   __syncthreads();
-  if (Tile<TS>::kSplit > 1) {
-    for (int e = tid; e < H * (TS / 4); e += kThr) {
-      const int j = e / (TS / 4), s = 4 * (e % (TS / 4));
-      float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  for (int e = tid; e < H * (TS / 4); e += kThr) {
+    const int j = e / (TS / 4), s = 4 * (e % (TS / 4));
+    float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-      for (int q = 0; q < Tile<TS>::kSplit; ++q) {
-        const float4 v = *reinterpret_cast<const float4*>(&S.part[q][j][s]);
-        z[0] += v.x; z[1] += v.y; z[2] += v.z; z[3] += v.w;
-      }
-      if (s < live) activate4<kGrad>(z, &out[j][s], kGrad ? &slope[j][s] : nullptr);
+    for (int q = 0; q < Tile<TS>::kSplit; ++q) {
+      const float4 v = *reinterpret_cast<const float4*>(&S.part[q][j][s]);
+      z[0] += v.x; z[1] += v.y; z[2] += v.z; z[3] += v.w;
     }
-    __syncthreads();
+    if (s < live) activate4<kGrad>(z, &out[j][s], kGrad ? &slope[j][s] : nullptr);
   }
+  __syncthreads();
 }
 
 // delta of the layer below: slope <- (W^T delta) * slope
@@ -307,39 +290,28 @@ template <int TS>
 __device__ __forceinline__ void back_delta(Smem<TS>& S, const __nv_bfloat16 (*wt)[kWRow],
                                            const float (*delta)[Tile<TS>::kRow],
                                            float (*slope)[Tile<TS>::kRow]) {
-  static_assert(Tile<TS>::kSpw == 4, "training tiles");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int sg = warp % Tile<TS>::kSg, part = warp / Tile<TS>::kSg;
   f2 acc[4][2];
 #pragma unroll
   for (int r = 0; r < 4; ++r) acc[r][0] = acc[r][1] = 0ull;
   product_backward<TS>(wt, delta, sg, part, acc);
-  if (Tile<TS>::kSplit == 1) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      float4* p = reinterpret_cast<float4*>(&slope[lane + 32 * r][4 * sg]);
-      const float4 g = *p;
-      *p = make_float4(lo2(acc[r][0]) * g.x, hi2(acc[r][0]) * g.y, lo2(acc[r][1]) * g.z,
-                       hi2(acc[r][1]) * g.w);
+  for (int r = 0; r < 4; ++r)
+    *reinterpret_cast<ulonglong2*>(&S.part[part][lane + 32 * r][4 * sg]) =
+        make_ulonglong2(acc[r][0], acc[r][1]);
+  __syncthreads();
+  for (int e = tid; e < H * (TS / 4); e += kThr) {
+    const int k = e / (TS / 4), s = 4 * (e % (TS / 4));
+    float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int q = 0; q < Tile<TS>::kSplit; ++q) {
+      const float4 v = *reinterpret_cast<const float4*>(&S.part[q][k][s]);
+      z.x += v.x; z.y += v.y; z.z += v.z; z.w += v.w;
     }
-  } else {
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-      *reinterpret_cast<ulonglong2*>(&S.part[part][lane + 32 * r][4 * sg]) =
-          make_ulonglong2(acc[r][0], acc[r][1]);
-    __syncthreads();
-    for (int e = tid; e < H * (TS / 4); e += kThr) {
-      const int k = e / (TS / 4), s = 4 * (e % (TS / 4));
-      float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll
-      for (int q = 0; q < Tile<TS>::kSplit; ++q) {
-        const float4 v = *reinterpret_cast<const float4*>(&S.part[q][k][s]);
-        z.x += v.x; z.y += v.y; z.z += v.z; z.w += v.w;
-      }
-      float4* p = reinterpret_cast<float4*>(&slope[k][s]);
-      const float4 g = *p;
-      *p = make_float4(z.x * g.x, z.y * g.y, z.z * g.z, z.w * g.w);
-    }
+    float4* p = reinterpret_cast<float4*>(&slope[k][s]);
+    const float4 g = *p;
+    *p = make_float4(z.x * g.x, z.y * g.y, z.z * g.z, z.w * g.w);
   }
   __syncthreads();
 }
