@@ -408,8 +408,7 @@ __device__ __forceinline__ void fused_field_prefix(FusedShared& S, long long* rh
 // already, are binned again, kRebin at a time into sum (plain, not padded), and
 // the block's node charge is written once more.  Replenishment adds a particle
 // per absorbed ion, so nothing the route kernel could check bounds a diode's
-// growth over its steps.  Out of line, and after the node charge of the normal
-// case: added to it there, the sum cost every step 0.15 of 10.2 us.
+// growth over its steps.
 constexpr int kRebin = kHistMaxParticles / 2;
 
 __device__ __noinline__ void fused_rebin(const DevState& st, const FusedShared& S, unsigned* hE,
@@ -471,7 +470,11 @@ __device__ __noinline__ void fused_rebin(const DevState& st, const FusedShared& 
   }
 }
 
-__global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_steps) {
+// kRebins: a diode's room and its replenishment let a block outgrow its
+// histograms within a launch (set_fused_shape).  A template, since the test
+// alone cost every step of the others 0.1 of 10 us.
+template <bool kRebins>
+__device__ __forceinline__ void fused_body(const DevState& st, int n_steps) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ FusedShared S;
   cg::cluster_group cl = cg::this_cluster();
@@ -597,7 +600,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
         node[j] = v;
       }
     }
-    if (4 * (hi - lo) + S.nemit > kHistMaxParticles)
+    if (kRebins && 4 * (hi - lo) + S.nemit > kHistMaxParticles)
       fused_rebin(st, S, hE, hI, rho_s, node, warp_field ? mn : 0, lo, hi);
     if (warp < 3) {
       const int x = lane < kFusedWarps ? S.wcnt[warp][lane] : 0;
@@ -805,7 +808,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
       dyn->step = S.step;
       dyn->next_id = S.base_id;
       dyn->pushed += S.pushed;
-      st.post[inst].fused_steps += (uint32_t)n_steps;
       dyn->win_steps += S.win_steps;
       dyn->emitted += S.emitted;
       dyn->replenished += S.replenished;
@@ -822,6 +824,13 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
   cl.sync();                           // no block leaves while its shared memory is read
 }
 
+__global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_steps) {
+  fused_body<false>(st, n_steps);
+}
+__global__ void __launch_bounds__(kFusedThreads, 1) k_fused_rebins(DevState st, int n_steps) {
+  fused_body<true>(st, n_steps);
+}
+
 // Which way the next steps run: 1 (the fused kernel) if its estimated time per
 // step is the smaller.
 // The fused kernel's histograms hold kHistMaxParticles per block, and a block
@@ -830,7 +839,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fused(DevState st, int n_s
 // over the steps; replenishment comes on top) would pass that, nor where the
 // expected candidates come near the size of the three kernels' buffer, whose
 // overflow is an error.
-__global__ void k_route(DevState st, int C, int sms, long long growth,
+__global__ void k_route(DevState st, int C, int sms, long long growth, int n_steps,
                         cudaGraphConditionalHandle handle) {
   __shared__ float ws[6][32];
   float longest = 0.0f, most = 0.0f, emit = 0.0f, sum = 0.0f, cands = 0.0f, total = 0.0f;
@@ -893,6 +902,7 @@ __global__ void k_route(DevState st, int C, int sms, long long growth,
     const StepEstimate e = estimate_step(st.n_inst, longest, sum, total, cands, emit, C, sms);
     const bool one = e.fused < e.three && 2.0f * cands + 4096.0f < (float)st.cand_cap &&
                      (long long)most + growth < (long long)kHistMaxParticles;
+    if (one) st.post[0].fused_steps += (uint32_t)n_steps;
     cudaGraphSetConditional(handle, one ? 1u : 0u);
   }
 }

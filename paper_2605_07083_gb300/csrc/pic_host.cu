@@ -28,7 +28,8 @@ __global__ void k_mid(DevState st);
 __global__ void k_mid_many(DevState st);
 __global__ void k_post(DevState st);
 __global__ void k_fused(DevState st, int n_steps);
-__global__ void k_route(DevState st, int C, int sms, long long growth,
+__global__ void k_fused_rebins(DevState st, int n_steps);
+__global__ void k_route(DevState st, int C, int sms, long long growth, int n_steps,
                         cudaGraphConditionalHandle handle);
 size_t fused_smem_bytes(int nodes);
 __global__ void k_field(DevState st);
@@ -410,14 +411,17 @@ cudaError_t raise_smem_limits(int device) {
                        (const void*)k_push_wide_many,
                        (const void*)k_deposit, (const void*)k_field,
                        (const void*)k_post, (const void*)k_profile, (const void*)k_phi,
-                       (const void*)k_mid, (const void*)k_mid_many, (const void*)k_fused};
+                       (const void*)k_mid, (const void*)k_mid_many, (const void*)k_fused,
+                       (const void*)k_fused_rebins};
   for (const void* f : fns) {
     e = set_dynamic_smem_limit(f, optin);
 
     if (e != cudaSuccess) return e;
   }
-  e = cudaFuncSetAttribute((const void*)k_fused, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
+  for (const void* f : {(const void*)k_fused, (const void*)k_fused_rebins}) {
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
   e = sort_prepare(optin);
   if (e == cudaSuccess && device >= 0 && device < 64) done[device] = true;
   return e;
@@ -716,6 +720,22 @@ void enqueue_steps(pic_handle* h, int n, int first) {
   }
 }
 
+// A block bins a diode's particles, its share of them, in 32-bit counters.  What
+// k_route checks bounds a diode's growth by emission and ionisation; where
+// replenishment can fill more room than a block's counters hold, the kernel
+// that looks at every step.
+void (*fused_kernel(const pic_handle* h))(DevState, int) {
+  bool rebins = false;
+  for (int i = 0; i < h->n_inst; ++i) {
+    int64_t room = 0;
+    for (int s = 0; s < 3; ++s) room += h->seg_cap[3 * i + s];
+    // a block's quads (three segments end in partial ones) and a step's emission
+    const int64_t most = room / h->fused_c + 16 + h->ic[i].emit_floor + 1;
+    rebins |= h->ic[i].replenish && most >= kHistMaxParticles;
+  }
+  return rebins ? k_fused_rebins : k_fused;
+}
+
 cudaError_t enqueue_fused(pic_handle* h, int n) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(h->n_inst * h->fused_c));
@@ -728,7 +748,7 @@ cudaError_t enqueue_fused(pic_handle* h, int n) {
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_fused, h->st, n);
+  return cudaLaunchKernelEx(&cfg, fused_kernel(h), h->st, n);
 }
 
 // Blocks per diode of k_fused: as many as let all clusters be resident at
@@ -751,7 +771,7 @@ void set_fused_shape(pic_handle* h) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_fused, &cfg) == cudaSuccess &&
+    if (cudaOccupancyMaxActiveClusters(&n, k_fused_rebins, &cfg) == cudaSuccess &&
         n >= (c > 1 ? h->n_inst : 1))
       h->fused_c = c;
   }
@@ -800,7 +820,7 @@ int add_routed_steps(pic_handle* h, cudaGraph_t g, int n, cudaGraphNode_t* tail)
   for (const InstConst& k : h->ic)
     growth = std::max(growth, (long long)n * (k.emit_floor + 1 + 2 * kEvCap));
   int C = h->fused_c, sms = h->sm_count;
-  void* args[] = {&h->st, &C, &sms, &growth, &cond};
+  void* args[] = {&h->st, &C, &sms, &growth, &n, &cond};
   cudaKernelNodeParams kp = {};
   kp.func = (void*)k_route;
   kp.gridDim = dim3(1);
@@ -1362,7 +1382,7 @@ int pic_diagnostics(pic_handle* h, int instance, pic_diag* out) {
 int pic_fused_steps(pic_handle* h, int64_t* steps) {
   if (!h || !steps) return PIC_EINVAL;
   OnDevice on(h);
-  k_read<<<1, 256, 0, h->stream>>>(h->st, 0, h->rb);
+  k_read<<<1, 256, 0, h->stream>>>(h->st, kReadFused, h->rb);
   int rc = read_done(h);
   if (rc != PIC_OK) return rc;
   *steps = (int64_t)h->rb->fused_steps;

@@ -145,7 +145,7 @@ struct InstDyn {
 struct PostScratch {
   int D[3], N[3];
   uint32_t base_id;
-  uint32_t fused_steps;              // steps that k_fused has run
+  uint32_t fused_steps;              // steps that k_fused has run (diode 0's entry)
   int route_n;                       // live particles, next id and step at k_route's last decision
   uint32_t route_id;
   long long route_step;
@@ -164,6 +164,7 @@ struct Readback {
   uint32_t fused_steps;    // PostScratch
   InstDyn dyn;
 };
+constexpr int kReadFused = -2;           // k_read's instance for the steps of k_fused
 constexpr size_t kReadNodes = 1024;
 constexpr size_t kReadBytes = kReadNodes + (size_t)(kMaxNz + 1) * 20;   // rho, phi (8 B), E
 static_assert(sizeof(Readback) <= kReadNodes && sizeof(InstDyn) % 4 == 0, "layout");

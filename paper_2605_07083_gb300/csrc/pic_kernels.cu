@@ -1200,15 +1200,16 @@ __device__ __forceinline__ void read_errors(const DevState& st, Readback* out) {
   if (threadIdx.x == 0) out->err = any;
 }
 
-// errors and, for inst >= 0, the diode's record and counts
+// errors and, for inst >= 0, the diode's record and counts; for kReadFused the
+// steps of k_fused
 __global__ void k_read(DevState st, int inst, Readback* out) {
   read_errors(st, out);
+  if (inst == kReadFused && threadIdx.x == 0) out->fused_steps = st.post[0].fused_steps;
   if (inst < 0) return;
   const int* src = reinterpret_cast<const int*>(st.dyn + inst);
   int* dst = reinterpret_cast<int*>(&out->dyn);
   for (int w = threadIdx.x; w < (int)(sizeof(InstDyn) / 4); w += blockDim.x) dst[w] = src[w];
   if (threadIdx.x < 3) out->count[threadIdx.x] = st.seg_count[3 * inst + threadIdx.x];
-  if (threadIdx.x == 0) out->fused_steps = st.post[inst].fused_steps;
 }
 
 // errors and the diode's fixed-point charge
