@@ -10,7 +10,6 @@
 #include <string.h>
 
 typedef struct { unsigned x, y, z; } dim3;
-typedef struct { int type, device; void* device_pointer; void* host_pointer; long reserved[8]; } Attributes;
 
 enum { kInvalidValue = 1, kInvalidResourceHandle = 400, kStreamDevice1 = 0x1000 };
 
@@ -38,28 +37,24 @@ int cudaDeviceGetAttribute(int* v, int attr, int device) {
 int cudaGetLastError(void) { int e = last_error; last_error = 0; return e; }
 const char* cudaGetErrorString(int e) { (void)e; return "fake"; }
 
-int cudaPointerGetAttributes(Attributes* a, const void* p) {
-  memset(a, 0, sizeof *a);
+/* cuPointerGetAttributes, for the five attributes in the order that the library asks for them */
+static int pointer_attributes(unsigned n, const int* what, void** data, unsigned long long p) {
+  static const int order[] = {2, 8, 9, 11, 12};   /* memory type, managed, device, range start, size */
+  if (n != 5 || memcmp(what, order, sizeof order)) return kInvalidValue;
+  *(unsigned*)data[0] = 0;
   for (int i = 0; i < entries; ++i)
-    if ((const char*)p >= table[i].p && (const char*)p < table[i].p + table[i].bytes) {
-      a->type = table[i].type;
-      a->device = table[i].device;
+    if ((const char*)(uintptr_t)p >= table[i].p && (const char*)(uintptr_t)p < table[i].p + table[i].bytes) {
+      *(unsigned*)data[0] = table[i].type == 0 ? 0 : 2;
+      *(int*)data[1] = table[i].type == 3;
+      *(int*)data[2] = table[i].device;
+      *(unsigned long long*)data[3] = (unsigned long long)(uintptr_t)table[i].p;
+      *(size_t*)data[4] = table[i].bytes;
     }
   return 0;
 }
-
-static int address_range(unsigned long long* base, size_t* bytes, unsigned long long p) {
-  for (int i = 0; i < entries; ++i)
-    if ((const char*)(uintptr_t)p >= table[i].p && (const char*)(uintptr_t)p < table[i].p + table[i].bytes) {
-      *base = (unsigned long long)(uintptr_t)table[i].p;
-      *bytes = table[i].bytes;
-      return 0;
-    }
-  return kInvalidValue;
-}
 int cudaGetDriverEntryPointByVersion(const char* name, void** fn, unsigned version, unsigned long long flags, int* found) {
   (void)version; (void)flags;
-  *fn = strcmp(name, "cuMemGetAddressRange") == 0 ? (void*)address_range : NULL;
+  *fn = strcmp(name, "cuPointerGetAttributes") == 0 ? (void*)pointer_attributes : NULL;
   *found = *fn ? 0 : 1;
   return 0;
 }
