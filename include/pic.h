@@ -377,7 +377,11 @@ int pic_sort_by_cell_static(const float* z, const float* vx, const float* vy, co
  * n_in, row-major) then b (n_out); the forward/backward read a bfloat16 copy
  * of it (same indices) for the weights and the FP32 biases, with FP32
  * activations and accumulation.  All pointers are device memory; work is
- * enqueued on cuda_stream; results are deterministic. */
+ * enqueued on cuda_stream; results are deterministic: the same arguments give
+ * the same bits.  The order of the FP32 sums, and with it the last bits of a
+ * sample's prediction or of a gradient, depends on the batch it is part of, for
+ * gradients also on the scratch offered (less than pic_mlp_scratch_bytes, down
+ * to one partial per 32 samples, selects larger tiles). */
 #define PIC_MLP_PARAMS 34308
 
 /* Scratch bytes pic_mlp_grad / pic_mlp_train_step need for a batch. */
