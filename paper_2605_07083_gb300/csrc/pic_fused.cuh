@@ -6,7 +6,7 @@
 // blocks, by how many diodes share the chip) owns a diode and runs n_steps of
 // it: field, constants, counts and tallies stay in shared memory, the
 // particles in L2, and the phases of a step meet at hardware cluster
-// barriers (9.4 us a step; 128 diodes of 5.5k particles 32.4 -> 11.4 us).  What
+// barriers (9.4 us a step; 128 diodes of 5.3k particles 32 -> 11.8 us).  What
 // is left is the phases' own round trips: about 40 % push, the rest lists, charge,
 // field and compaction, of which only latency counts; a block keeps its
 // registers below the limit, since a spilled one is fetched from L2 after

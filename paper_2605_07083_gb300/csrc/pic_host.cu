@@ -500,9 +500,9 @@ int set_launch_shape(pic_handle* h) {
   if (e != cudaSuccess) return cuda_fail(h, e);
   // many candidates: more expected per step (probability x capacity) than one
   // per thread of one k_mid block per SM.  Then the push writes records that
-  // spare k_mid three random reads each (paper scan, 1 % candidates: k_mid 29
-  // -> 22 us for 2 us more of the push); with few the records only cost the
-  // push registers (64-diode sweep: push 166 -> 171 us).
+  // spare k_mid three random reads each (paper scan, 1 % candidates: k_mid 7 us
+  // less for 2 us more of the push); with few the records only cost the push
+  // registers (64-diode sweep: push 166 -> 171 us).
   double cand = 0.0;
   for (int i = 0; i < h->n_inst; ++i)
     for (int s = 0; s < 3; ++s)
@@ -759,9 +759,10 @@ cudaError_t enqueue_fused(pic_handle* h, int n) {
 }
 
 // Blocks per diode of k_fused: as many as let all clusters be resident at
-// once, a power of two up to 16 (a cluster of 16, which has to be allowed,
-// takes 9.8 us for 22k particles and 15.4 for 135k, one of 8 10.4 and 18.4); 0
-// where a block does not fit (its shared memory grows with the cells).
+// once, a power of two up to 16 (a cluster of 16, which has to be allowed, took
+// 9.8 us for 22k particles and 15.4 for 135k where one of 8 took 10.4 and 18.4,
+// before the charge was summed by slices: 9.4); 0 where a block does not fit (its
+// shared memory grows with the cells).
 void set_fused_shape(pic_handle* h) {
   h->fused_c = 0;
   h->fused_smem = fused_smem_bytes(h->max_nodes);

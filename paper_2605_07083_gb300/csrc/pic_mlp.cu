@@ -36,8 +36,8 @@ static_assert(NP == PIC_MLP_PARAMS, "parameter count");
 // the partials' stores.  A 4 x 4 register tile needs two shared loads per 16
 // FMAs; with one thread per unit each FMA row had a 2-byte global load and a
 // scalar shared load per FMA, 150 us even for one tile.  Measured before and
-// after: training step of 4096 samples 161 -> 42 us, gradient of 100 samples
-// 154 -> 20.5 us, prediction of 41216 samples 287 -> 82 us.
+// after: training step of 4096 samples 161 -> 41 us, gradient of 100 samples
+// 154 -> 18.6 us, prediction of 41216 samples 287 -> 82 us.
 constexpr int kThr = 512, kWarps = kThr / 32;
 constexpr int kWRow = H + 8;                 // bfloat16 per row of a transposed matrix
 constexpr int kSms = 152;                    // tiles are kept to one wave while they fit
@@ -673,7 +673,7 @@ __device__ __forceinline__ float tree_sum(float (&x)[kRedUnroll]) {
 // four times as many partials as tiles of 32; one after another, 152 of them
 // have an error of up to 151 roundings of the sum, so 13.  Sixteen running sums
 // with one tree at the end are as exact, but left the compiler fewer loads in
-// flight: the training step of 4096 samples 45.2 us instead of 41.7.)
+// flight: the training step of 4096 samples 45.2 us instead of 41.0.)
 __global__ void k_mlp_reduce_adam(const float* part, const float* lpart,
                                   int n_part, long long batch, float* __restrict__ grad,
                                   float* __restrict__ loss, float* __restrict__ master,
