@@ -114,7 +114,9 @@ typedef struct pic_tuning {
                                  32; default: the size that keeps closest to 24 resident warps
                                  per SM for the handle's cell count, the first of 384, 256,
                                  128, 160, ... that does, or one block of 640..768 threads
-                                 per SM where the cell grid leaves two blocks too few) */
+                                 per SM where the cell grid leaves two blocks too few warps
+                                 and a diode has a million particles or more before the
+                                 first step) */
     int32_t push_blocks_per_sm;  /* cap on resident blocks per SM (default: occupancy limit) */
     int32_t sort_period;      /* counting sort by cell every this many steps; < 0 disables */
     int32_t graph_steps;      /* longest step loop captured as one CUDA graph (default 64,

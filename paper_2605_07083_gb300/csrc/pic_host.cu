@@ -110,6 +110,8 @@ struct pic_handle {
   std::vector<uint32_t> known_id;
   int bw_len = 0;
   int mcc_blocks = 0;
+  bool wide_ok = true;          // the push may take one wide block per SM (wide_pays)
+  bool wide_matters = false;    // and the cell grid leaves it the choice
   int fused_c = 0;              // blocks per diode of k_fused (0: not taken)
   size_t fused_smem = 0;
   bool sort_ready = false;
@@ -472,9 +474,10 @@ int push_warps(const pic_handle* h, int threads, int chunk) {
 // threads against 2 x 320 at 4096 cells, push 112 -> 107 us on the paper
 // scan.  With room for two blocks it is the slower one (64-diode sweep, 22
 // warps in two blocks against 24 in one: 166 and 170 us; production diode 44
-// and 45: all of a block's warps wait for its slowest).  A caller's choice of
-// either is kept.
+// and 45: all of a block's warps wait for its slowest), and so it is with few
+// particles (wide_pays).  A caller's choice of either is kept.
 void default_push_shape(pic_handle* h) {
+  h->wide_matters = false;
   int best_t = h->threads_set ? h->push_threads : 384;
   int best_c = h->chunk_set ? h->push_chunk : 64;
   int best_w = -1;
@@ -486,11 +489,33 @@ void default_push_shape(pic_handle* h) {
   };
   for (int c : {64, 32}) {
     for (int t : {384, 256, 128, 160, 192, 224, 288, 320, 352}) consider(t, c);
-    if (c == 64 && best_w < 20)
-      for (int t : {768, 736, 704, 672, 640}) consider(t, c);
+    if (c == 64 && best_w < 20) {
+      h->wide_matters = !h->threads_set;
+      if (h->wide_ok)
+        for (int t : {768, 736, 704, 672, 640}) consider(t, c);
+    }
   }
   h->push_threads = best_t;
   h->push_chunk = best_c;
+}
+
+// Does one wide push block per SM pay?  It starts and ends later than two
+// (a grid of 4096 cells: 16 instead of 13 us for 20k particles) and streams
+// faster, the more so the fewer segments a block meets.  Steps, two blocks and
+// one: 4096 cells, electrons of one diode: 400k 22.7 and 23.0 us, 1M 25.2 and
+// 24.4, 8M 51.8 and 47.1; paper diodes: one of 0.98M 27.2 and 28.6, of 2.05M
+// 32.3 and 31.1, 3 of 2.9M together 40.5 and 41.4, 11 of 1.8M 40.6 and 42.0, of
+// 5.4M 55.0 and 54.5, of 22M 132 and 126: from a million a diode on.  The
+// particles are those that the host knows of, or, in a handle without any, a
+// quarter of its room.
+bool wide_pays(const pic_handle* h) {
+  int64_t live = 0, room = 0;
+  for (int g = 0; g < h->n_seg; ++g) {
+    live += h->known_count[g];
+    room += h->seg_cap[g];
+  }
+  if (live == 0) live = room / 4;
+  return live >= 1000000LL * h->n_inst;
 }
 
 void set_fused_shape(pic_handle* h);
@@ -531,7 +556,9 @@ int set_launch_shape(pic_handle* h) {
   // ~10 us later on the paper scan)
   const int places = 2 * h->sm_count - 4 * h->n_inst * h->st.kp - 1;
   h->mcc_blocks = h->st.cand_many ? std::max(h->sm_count, places) : h->sm_count;
-  const size_t need = (size_t)h->n_seg * h->G;
+  // (room for two blocks per SM where their number may change, fit_push_shape)
+  const int room = h->wide_matters ? std::max(h->G, 2 * h->sm_count) : h->G;
+  const size_t need = (size_t)h->n_seg * room;
   if (need > h->dcount_ints) {
     void* p = dev_alloc(h, need * sizeof(int32_t));
     if (!p) return PIC_ENOMEM;
@@ -546,11 +573,11 @@ int set_launch_shape(pic_handle* h) {
   // first block ran about twice as fast as the third)
   // layout: bwp [G + 1] long long, bw [G] int, bt [G] int, bw_n [2] int
   const size_t bw_bytes = sizeof(long long) * (size_t)(2 * h->G + 2);
-  if (h->G > h->bw_len) {
-    void* p = dev_alloc(h, bw_bytes);
+  if (room > h->bw_len) {
+    void* p = dev_alloc(h, sizeof(long long) * (size_t)(2 * room + 2));
     if (!p) return PIC_ENOMEM;
     h->st.bwp = (long long*)p;
-    h->bw_len = h->G;
+    h->bw_len = room;
   }
   h->st.bw = (int*)(h->st.bwp + h->G + 1);
   h->st.bt = h->st.bw + h->G;
@@ -575,11 +602,11 @@ int set_launch_shape(pic_handle* h) {
     if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(h->stream);
     if (e2 != cudaSuccess) return cuda_fail(h, e2);
   }
-  if (h->G + 1 > h->bstart_len) {
-    void* p = dev_alloc(h, sizeof(int64_t) * (size_t)(h->G + 1));
+  if (room + 1 > h->bstart_len) {
+    void* p = dev_alloc(h, sizeof(int64_t) * (size_t)(room + 1));
     if (!p) return PIC_ENOMEM;
     h->st.bstart = (int64_t*)p;
-    h->bstart_len = h->G + 1;
+    h->bstart_len = room + 1;
   }
   // k_mid: a diode's charge and emission histogram, or a segment's piece
   // ranges and prefix; k_post: the staged absorbed list or the event keys
@@ -700,6 +727,16 @@ void set_profile_mode(pic_handle* h) {
 void launch_profile(pic_handle* h) {
   if (h->st.prof_period > 0)
     k_profile<<<dim3((unsigned)h->prof_gx, (unsigned)h->n_seg), 256, h->prof_smem, h->stream>>>(h->st);
+}
+
+// Before the first step of an injected or loaded state: the push shape by its
+// particles (wide_pays).  The results do not depend on the shape.
+int fit_push_shape(pic_handle* h) {
+  if (!h->wide_matters || !h->counts_known) return PIC_OK;
+  const bool pays = wide_pays(h);
+  if (pays == h->wide_ok) return PIC_OK;
+  h->wide_ok = pays;
+  return set_launch_shape(h);
 }
 
 // one time step; the sort, when due, follows the step
@@ -1143,6 +1180,7 @@ int pic_create(const pic_config* cfgs, int n_instances, void* cuda_stream,
   h->known_id.assign(h->n_inst, 0u);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) { pic_destroy(h); return PIC_ECUDA; }
+  h->wide_ok = wide_pays(h);
   int rc = set_launch_shape(h);
   if (rc != PIC_OK) { pic_destroy(h); return rc; }
   *out = h;
@@ -1302,7 +1340,8 @@ static int step_plan(pic_handle* h, int64_t n_steps, bool run) {
 int pic_step(pic_handle* h, int64_t n_steps) {
   if (!h || n_steps < 0) return PIC_EINVAL;
   if (h->sticky != PIC_OK) return h->sticky;
-  int rc = ensure_field(h);
+  int rc = fit_push_shape(h);
+  if (rc == PIC_OK) rc = ensure_field(h);
   if (rc != PIC_OK) return rc;
   return step_plan(h, n_steps, true);
 }
@@ -1310,7 +1349,8 @@ int pic_step(pic_handle* h, int64_t n_steps) {
 int pic_prepare_steps(pic_handle* h, int64_t n_steps) {
   if (!h || n_steps < 0) return PIC_EINVAL;
   if (h->sticky != PIC_OK) return h->sticky;
-  int rc = ensure_field(h);
+  int rc = fit_push_shape(h);
+  if (rc == PIC_OK) rc = ensure_field(h);
   if (rc != PIC_OK) return rc;
   return step_plan(h, n_steps, false);
 }
@@ -1318,7 +1358,8 @@ int pic_prepare_steps(pic_handle* h, int64_t n_steps) {
 int pic_profile_steps(pic_handle* h, int64_t n_steps, pic_profile* out) {
   if (!h || !out || n_steps < 0) return PIC_EINVAL;
   std::memset(out, 0, sizeof(*out));
-  int rc = ensure_field(h);
+  int rc = fit_push_shape(h);
+  if (rc == PIC_OK) rc = ensure_field(h);
   if (rc != PIC_OK) return rc;
   h->counts_known = false;
   std::vector<cudaEvent_t> ev(6 * (size_t)std::max<int64_t>(n_steps, 1));

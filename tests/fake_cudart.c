@@ -82,13 +82,14 @@ int cudaFuncSetAttribute(const void* f, int attr, int v) {
 }
 int cudaGetSymbolAddress(void** p, const void* s) { (void)s; static int word[4]; *p = word; return 0; }
 int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* f, int t, size_t m, unsigned fl) {
-  (void)f; (void)t; (void)m; (void)fl;
-  *n = 2;
+  (void)f; (void)fl;
+  const int by_memory = m ? (int)(227u * 1024u / m) : 32, by_registers = 65536 / (80 * t);
+  *n = by_memory < by_registers ? by_memory : by_registers;
   return 0;
 }
 int cudaOccupancyMaxActiveClusters(int* n, const void* f, const void* cfg) { (void)f; (void)cfg; *n = 8; return 0; }
 
-static struct { const void* f; const char* name; } kernels[256];
+static struct { const void* f; const char* name; int launches; } kernels[256];
 static int n_kernels = 0;
 const char* fake_last_kernel = "";
 
@@ -99,8 +100,17 @@ static int launch(const void* f, void* stream) {
   }
   ++fake_launches;
   for (int i = 0; i < n_kernels; ++i)
-    if (kernels[i].f == f) fake_last_kernel = kernels[i].name;
+    if (kernels[i].f == f) {
+      fake_last_kernel = kernels[i].name;
+      ++kernels[i].launches;
+    }
   return 0;
+}
+int fake_count(const char* part) {                  /* launches of the kernels with that in their name */
+  int n = 0;
+  for (int i = 0; i < n_kernels; ++i)
+    if (strstr(kernels[i].name, part)) n += kernels[i].launches;
+  return n;
 }
 static void* pushed_stream;
 unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t m, void* s) {

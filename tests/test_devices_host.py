@@ -146,3 +146,32 @@ for _ in range(40):
 assert word("fake_graph_launches").value > 0 and captures > 0
 assert word("fake_captures").value == captures
 ''')
+
+
+@pytest.mark.parametrize("cells,room,live,tune,wide", [
+    (4096, 3 << 20, 20000, {}, False), (4096, 3 << 20, 900000, {}, False),
+    (4096, 3 << 20, 1100000, {}, True), (4096, 3 << 20, 0, {}, False),
+    (4096, 1 << 23, 0, {}, True), (4096, 1 << 23, 20000, {}, False),
+    (4096, 3 << 20, 1100000, {"push_threads": 320}, False), (2048, 3 << 20, 1100000, {}, False)])
+def test_one_wide_push_block_only_for_many_particles(run, cells, room, live, tune, wide):
+    """The grids that leave two push blocks too few warps take one wide block
+    per SM from a million particles on; the first step after an injection
+    decides, and by the room where there are none."""
+    run(f'''
+h = C.c_void_p()
+word("fake_device").value = 1
+p = dict(W.single_diode_production(), Nz={cells}, capacity=({room} // 3,) * 3)
+cfg = pic.make_config(p)
+assert lib.pic_create(C.byref(cfg), 1, C.c_void_p(0x1000), None, C.byref(h)) == 0
+t = pic.PicTuning(size=C.sizeof(pic.PicTuning), graph_steps=-1, **{tune})
+assert lib.pic_tune(h, C.byref(t)) == 0
+for sp in (0, 1):
+    if {live}:
+        a = [(C.c_float * ({live} // 2))() for _ in range(4)]
+        assert lib.pic_inject(h, 0, sp, {live} // 2, *a, 0) == 0
+for _ in range(3):
+    assert lib.pic_step(h, 2) == 0
+fake.fake_count.argtypes = [C.c_char_p]
+steps, one = fake.fake_count(b"k_post"), fake.fake_count(b"k_push_wide")
+assert steps == 6 and one == (6 if {wide} else 0)
+''')

@@ -5,8 +5,10 @@ fused kernel of small diodes.  GPU.
 
 Many candidates: a probability of 2 % of room for 3 x 2^21 particles, above one
 per thread of a block per SM, selects the kernels whose candidate records carry
-the particle.  4096 cells leave 64-quad chunks room for one wide block per SM,
-which is the default there; a chosen size or chunk selects the others."""
+the particle; 0.5 % do not.  4096 cells leave 64-quad chunks room for one wide
+block per SM, the default for that room as long as the live counts are not
+known before a step: the particles come after a first, empty step.  A chosen
+size or chunk selects the others."""
 import numpy as np
 import pytest
 
@@ -33,10 +35,10 @@ def test_results_do_not_depend_on_the_push_shape(pic, cells, many):
     p = W.single_diode_small(seed=61) if cells == 128 else W.single_diode_production(seed=62)
     # the probability at the energy bound, of electrons
     g = np.sqrt(2 * p["E_cap_e_eV"] * W.E_CHARGE / W.M_E)
-    prob = 0.02
+    prob = 0.02 if many else 0.005
     p.update(Nz=cells, replenish=1, window_start=2,
              n_gas=-np.log1p(-prob) / (p["sigma_el_e"] * g * p["dt"]),
-             capacity=(1 << 21,) * 3 if many else (65536,) * 3)
+             capacity=(1 << 21,) * 3)
     st = mixed_state(p, 63, 30001, 10003)
     shapes = [{}, {"push_threads": 128}, {"push_threads": 320}, {"push_chunk": 32},
               {"push_threads": 160, "push_chunk": 32}, {"push_blocks_per_sm": 1}]
@@ -44,13 +46,14 @@ def test_results_do_not_depend_on_the_push_shape(pic, cells, many):
     for shape in shapes:
         d = pic.Diode(p)
         d.tune(graph_steps=-1, **shape)
+        d.step(1)
         for sp in range(3):
             d.inject(sp, *st[sp])
         d.step(12)
         runs.append(([d.state(sp) for sp in range(3)], d.rho_fixed(), d.diagnostics()))
         d.close()
     sa, ra, da = runs[0]
-    assert da["candidates"].sum() > 3000 and da["count"].sum() > 0
+    assert da["candidates"].sum() > 1000 and da["count"].sum() > 0
     for (sb, rb, db), shape in zip(runs[1:], shapes[1:]):
         assert np.array_equal(ra, rb), shape
         for x, y in zip(sa, sb):
