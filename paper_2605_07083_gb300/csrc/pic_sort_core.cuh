@@ -11,10 +11,10 @@
 //
 // What bounds it: 44 B per particle (z twice, the other fields and the output
 // once), so HBM for a set larger than L2; below ~1e5 particles the four
-// dependent launches.  4M particles over 2048 cells in random order: 101 us
-// (1.7 TB/s), 930 us before, of which the prefix took 865 us in one block and
-// the scatter 261 us; the handle's sort of 2.1M particles 92 us with its copy
-// back, 320 us before.
+// dependent launches.  4M particles over 2048 cells in random order: 91 us
+// (1.9 TB/s), 930 us before, of which the prefix took 865 us in one block and
+// the scatter 261 us; the handle's sort of 2.1M particles 75 us with its copy
+// back, 320 us before.  A set of one chunk needs the scatter alone.
 //   * The prefix runs over all entries of the histogram: a block per tile of
 //     4096 entries, ~4 us for the sums and ~5 us for the prefix (each block
 //     adds up the sums of the tiles before its own).
@@ -22,7 +22,7 @@
 //     store.  Through shared memory a chunk is first put in cell order, one
 //     field at a time, so a warp writes a few runs; the longer the chunk the
 //     longer the runs (at 2048 cells 4 particles per run in chunks of 8192:
-//     135 us; 6.5 in chunks of 13.3k: 80 us).  What is left of the scatter is
+//     135 us; 6.5 in chunks of 13.3k: 80 us, both with spilled registers).  What is left of the scatter is
 //     those partial lines: with contiguous writes the same kernel took 30 %
 //     less.
 //   * A warp ranks its 32 particles without __match_any_sync (about 50 clocks
@@ -209,7 +209,9 @@ __device__ __forceinline__ void sort_scatter(const View& v, int c, unsigned char
 #pragma unroll
   for (int k = 0; k < kItems; ++k)
     x[k] = k < nk ? __float_as_uint(v.z[c0 + w0 + lane + 32 * k]) : 0u;
-  for (int j = tid; j < Nz; j += kThr) delta[j] = v.hist[(long long)j * v.nch + c];
+  // with one column in all, the place within the chunk is the place
+  const bool whole = v.nch == 1;
+  for (int j = tid; j < Nz; j += kThr) delta[j] = whole ? 0 : v.hist[(long long)j * v.nch + c];
   for (int k = tid; k < kWarps * Nze / 2; k += kThr) reinterpret_cast<uint32_t*>(cnt)[k] = 0u;
   __syncthreads();
   // ---- cells and ranks: key[k] = (cell << 16) | rank among the warp's equals
@@ -301,7 +303,7 @@ __device__ __forceinline__ void sort_scatter(const View& v, int c, unsigned char
 #pragma unroll
   for (int k = 0; k < kItems; ++k) {
     const int s = k * kThr + tid;
-    to[k] = s < total ? delta[cell_s[s]] + s : 0;
+    to[k] = s < total ? (whole ? s : delta[cell_s[s]] + s) : 0;
   }
   // ---- the fields, through two stages in turn: the next field's loads are
   // in flight while this one is written (a rolled loop: unrolled, the

@@ -123,9 +123,13 @@ extern "C" int pic_sort_by_cell_static(const float* z, const float* vx, const fl
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const unsigned tiles =
       (unsigned)(((long long)n_cells * nch + sortcore::kTile - 1) / sortcore::kTile);
-  k_static_hist<<<(unsigned)nch, kThreads, n_cells * sizeof(int), s>>>(v);
-  k_static_tilesum<<<tiles, kThreads, 0, s>>>(v);
-  k_static_scan<<<tiles, kThreads, 0, s>>>(v);
+  // up to a column's particles the scatter alone is the sort: 100 particles over
+  // 128 cells take 13 us, with the histogram and its prefix 29
+  if (nch > 1) {
+    k_static_hist<<<(unsigned)nch, kThreads, n_cells * sizeof(int), s>>>(v);
+    k_static_tilesum<<<tiles, kThreads, 0, s>>>(v);
+    k_static_scan<<<tiles, kThreads, 0, s>>>(v);
+  }
   const size_t smem = sortcore::scatter_smem(n_cells, warps);
   if (warps == 32) k_static_scatter<32><<<(unsigned)nch, 1024, smem, s>>>(v);
   else k_static_scatter<16><<<(unsigned)nch, 512, smem, s>>>(v);
