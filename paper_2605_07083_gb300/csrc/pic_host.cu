@@ -1627,9 +1627,14 @@ size_t ckpt_bytes(const pic_handle* h, const std::vector<int32_t>& counts, bool 
   return b;
 }
 
+// the live counts, and the error bits for flags_of: one wait for both
 int read_counts(pic_handle* h, std::vector<int32_t>& counts) {
+  OnDevice on(h);
   counts.resize(h->n_seg);
-  cudaError_t e = cudaMemcpyAsync(counts.data(), h->st.seg_count, sizeof(int32_t) * h->n_seg,
+  k_read<<<1, 256, 0, h->stream>>>(h->st, -1, h->rb);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(counts.data(), h->st.seg_count, sizeof(int32_t) * h->n_seg,
                                   cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   return e == cudaSuccess ? PIC_OK : cuda_fail(h, e);
@@ -1643,7 +1648,7 @@ int pic_checkpoint_bytes(pic_handle* h, size_t* bytes) {
   int rc = read_counts(h, counts);
   if (rc != PIC_OK) return rc;
   *bytes = ckpt_bytes(h, counts, h->st.phi_sum != nullptr);
-  return check_flags(h);
+  return flags_of(h);
 }
 
 int pic_save(pic_handle* h, void* host_buf, size_t bytes, size_t* written) {
@@ -1702,7 +1707,7 @@ int pic_save(pic_handle* h, void* host_buf, size_t bytes, size_t* written) {
   if (e != cudaSuccess) return cuda_fail(h, e);
   std::memcpy(dyn_at, dyn.data(), sizeof(InstDyn) * h->n_inst);
   if (written) *written = (size_t)(p - (char*)host_buf);
-  return check_flags(h);
+  return flags_of(h);
 }
 
 int pic_load(pic_handle* h, const void* host_buf, size_t bytes) {
@@ -1835,10 +1840,7 @@ const char* pic_last_error(const pic_handle* h) {
 }
 
 int pic_synchronize(pic_handle* h) {
-  if (!h) return PIC_EINVAL;
-  cudaError_t e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  return check_flags(h);
+  return h ? check_flags(h) : PIC_EINVAL;     // reads the errors behind all work, and waits
 }
 
 void pic_destroy(pic_handle* h) {
