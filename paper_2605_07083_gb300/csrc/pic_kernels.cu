@@ -1762,14 +1762,22 @@ __global__ void __launch_bounds__(kPostThreads, 2) k_post(DevState st) {
   constexpr int kEmitRegs = 2;
   float ez[kEmitRegs], evx[kEmitRegs], evy[kEmitRegs], evz[kEmitRegs];
   bool have_emit = false;
+  const auto draw_first = [&]() {
+    const int Ne = emitted_count(ic, step);
+#pragma unroll
+    for (int j = 0; j < kEmitRegs; ++j)
+      if (tid + j * nt < Ne)
+        emitted_electron(ic, tid + j * nt, step, ez[j], evx[j], evy[j], evz[j]);
+    have_emit = true;
+  };
   if (D > 0) {
     const int h = lower_bound(dd, D, Nn);        // holes: the listed slots below Nn
-    {
+    if (D <= nt) {                               // a slot per thread
       const int k = tid, t0 = Nn + k;
       int to = -1;
       float z, vx, vy, vz;
       uint32_t id;
-      if (k < D && D <= nt) {
+      if (k < D) {
         const int a2 = lower_bound(dd, D, t0);   // listed slots before the tail slot
         if (a2 == D || (int)dd[a2] != t0) {
           to = (int)dd[k - (a2 - h)];            // the hole of the same rank
@@ -1781,49 +1789,43 @@ __global__ void __launch_bounds__(kPostThreads, 2) k_post(DevState st) {
           id = st.id[src];
         }
       }
-      if (sp == 0) {
-        const int Ne = emitted_count(ic, step);
-#pragma unroll
-        for (int j = 0; j < kEmitRegs; ++j)
-          if (tid + j * nt < Ne)
-            emitted_electron(ic, tid + j * nt, step, ez[j], evx[j], evy[j], evz[j]);
-        have_emit = true;
-      }
+      if (sp == 0) draw_first();
       if (to >= 0) put_particle(st, off, to, z, vx, vy, vz, id);
-    }
-    // more than nt, four in a row per thread: one search and one round trip for
-    // all of them (one slot per thread and round took 540 instead of 359 us for
-    // 100000 absorbed, whose list the search reads from L2)
-    constexpr int kPer = 4;
-    for (int base = 0; D > nt && base < D; base += kPer * nt) {
-      const int k0 = base + kPer * tid;
-      if (k0 >= D) continue;
-      int a2 = lower_bound(dd, D, Nn + k0);
-      int next = a2 < D ? (int)dd[a2] : INT_MAX;       // the listed slot at or after the tail slot
-      int to[kPer];
-      float z[kPer], vx[kPer], vy[kPer], vz[kPer];
-      uint32_t id[kPer];
+    } else {
+      // four in a row per thread: one search and one round trip for all of them
+      // (one slot per thread and round took 540 instead of 359 us for 100000
+      // absorbed, whose list the search reads from L2)
+      constexpr int kPer = 4;
+      for (int base = 0; base < D; base += kPer * nt) {
+        const int k0 = base + kPer * tid;
+        int a2 = k0 < D ? lower_bound(dd, D, Nn + k0) : D;
+        int next = a2 < D ? (int)dd[a2] : INT_MAX;     // the listed slot at or after the tail slot
+        int to[kPer];
+        float z[kPer], vx[kPer], vy[kPer], vz[kPer];
+        uint32_t id[kPer];
 #pragma unroll
-      for (int u = 0; u < kPer; ++u) {
-        to[u] = -1;
-        const int t0 = Nn + k0 + u;
-        if (k0 + u >= D) continue;
-        if (next == t0) {
-          ++a2;
-          next = a2 < D ? (int)dd[a2] : INT_MAX;
-        } else {
-          to[u] = (int)dd[k0 + u - (a2 - h)];
-          const long long src = off + t0;
-          z[u] = st.z[src];
-          vx[u] = st.vx[src];
-          vy[u] = st.vy[src];
-          vz[u] = st.vz[src];
-          id[u] = st.id[src];
+        for (int u = 0; u < kPer; ++u) {
+          to[u] = -1;
+          const int t0 = Nn + k0 + u;
+          if (k0 + u >= D) continue;
+          if (next == t0) {
+            ++a2;
+            next = a2 < D ? (int)dd[a2] : INT_MAX;
+          } else {
+            to[u] = (int)dd[k0 + u - (a2 - h)];
+            const long long src = off + t0;
+            z[u] = st.z[src];
+            vx[u] = st.vx[src];
+            vy[u] = st.vy[src];
+            vz[u] = st.vz[src];
+            id[u] = st.id[src];
+          }
         }
-      }
+        if (sp == 0 && base == 0) draw_first();
 #pragma unroll
-      for (int u = 0; u < kPer; ++u)
-        if (to[u] >= 0) put_particle(st, off, to[u], z[u], vx[u], vy[u], vz[u], id[u]);
+        for (int u = 0; u < kPer; ++u)
+          if (to[u] >= 0) put_particle(st, off, to[u], z[u], vx[u], vy[u], vz[u], id[u]);
+      }
     }
   }
   __syncthreads();                   // tail slots are read, shared memory is reused below
