@@ -666,6 +666,15 @@ __device__ __forceinline__ float tree_sum(float (&x)[kRedUnroll]) {
   return x[0];
 }
 
+// s += x, the rounding error of that into low (Knuth's two-sum).  One number's
+// error does not average out as a gradient's does, and a 64-bit sum, whose
+// dependent additions take ~150 clocks each, made the kernel end 2 us later.
+__device__ __forceinline__ void add_exactly(float& s, float& low, float x) {
+  const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+  low += __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+  s = t;
+}
+
 // grad[p] = sum over CTAs of the partials; optional Adam update of the FP32
 // master with the bfloat16 copy re-rounded (Kingma & Ba 2015).  The order is
 // fixed: a tree over sixteen partials, the trees one after another.  (The tiles
@@ -686,10 +695,14 @@ __global__ void k_mlp_reduce_adam(const float* part, const float* lpart,
   // loads: they change during this kernel's life, so no __restrict__ const)
   cudaGridDependencySynchronize();
   if (p >= kRedBlocks * kRedThreads - 32 && loss) {     // a warp without parameters
-    float L = 0.0f;
-    for (int b = threadIdx.x & 31; b < n_part; b += 32) L += lpart[b];
-    for (int off = 16; off > 0; off >>= 1) L += __shfl_down_sync(0xffffffffu, L, off);
-    if ((threadIdx.x & 31) == 0) *loss = L / (float)(batch * OUT);
+    float L = 0.0f, low = 0.0f;                // the sum and what its roundings dropped
+    for (int b = threadIdx.x & 31; b < n_part; b += 32) add_exactly(L, low, lpart[b]);
+    for (int off = 16; off > 0; off >>= 1) {
+      const float other = __shfl_down_sync(0xffffffffu, L, off);
+      low += __shfl_down_sync(0xffffffffu, low, off);
+      add_exactly(L, low, other);
+    }
+    if ((threadIdx.x & 31) == 0) *loss = (L + low) / (float)(batch * OUT);
   }
   if (p >= NP) return;
   float gsum = 0.0f;
